@@ -154,6 +154,16 @@ struct FusionList {
     int* refresh_tile = nullptr;  // tiles to refresh
 };
 
+// Where the ray cast can meet the surface: one bit per brick of 8^3 cells,
+// set when some cell of the brick has a corner whose value was ever fused or
+// uploaded as zero or negative (never cleared but by a reset or an upload, so
+// a set bit may be stale; a clear one is certain).  A 64-bit word holds 4^3
+// bricks (32^3 cells): 32 KB at 512^3, small enough to stay in L1.
+struct SurfaceMap {
+    unsigned long long* words = nullptr;
+    int wx = 0, wy = 0, wz = 0;  // words per axis: ceil(n / 32)
+};
+
 struct pf_volume {
     pf_volume_desc desc;
     int device = 0;
@@ -168,6 +178,7 @@ struct pf_volume {
     int fitness_variant = 0;
     pf_status last_status = PF_OK;  // last failing status of a call on this volume
     FusionList list;
+    SurfaceMap surf;
     pf_workspace ws;
 };
 
@@ -272,4 +283,25 @@ inline CamK make_cam(const pf_intrinsics* in)
 __device__ inline bool pf_depth_usable(float z, float dmin, float dmax)
 {
     return isfinite(z) && z >= dmin && z <= dmax;
+}
+
+// Marks the bricks that hold a cell with one of these nodes as a corner: the
+// warp's lane l stands for node (i0 + l, j, k0 ... k0 + 7), i0 a multiple of
+// 32 and k0 of 8; bit l of any is set when one of its eight nodes is zero or
+// negative, bit l of first when the one at k0 is.  Called by a whole warp.
+__device__ inline void pf_mark_surface(const SurfaceMap& s, unsigned any, unsigned first, int i0, int j, int k0)
+{
+    if (any == 0u) return;
+    // lanes 0..19: bricks i0/8 + q (q = -1..3) x (j/8 or the one below) x (k0/8 or the one below)
+    const int lane = threadIdx.x & 31;
+    const int q = lane % 5 - 1, below_y = (lane / 5) & 1, below_z = lane / 10;
+    if (lane >= 20 || (below_y && (j & 7) != 0)) return;
+    const unsigned m = below_z ? first : any;
+    // a brick's cells reach the first node of the next brick
+    const unsigned nodes = q < 0 ? m & 1u : (m >> (8 * q)) & 0x1ffu;
+    const int bx = (i0 >> 3) + q, by = (j >> 3) - below_y, bz = (k0 >> 3) - below_z;
+    if (nodes == 0u || bx < 0 || by < 0 || bz < 0) return;
+    unsigned long long* w = s.words + (bx >> 2) + (size_t)s.wx * ((by >> 2) + (size_t)s.wy * (bz >> 2));
+    const unsigned long long bit = 1ull << ((bx & 3) | ((by & 3) << 2) | ((bz & 3) << 4));
+    if ((__ldcg(w) & bit) == 0ull) atomicOr(w, bit);
 }

