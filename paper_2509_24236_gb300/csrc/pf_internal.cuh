@@ -142,16 +142,22 @@ struct pf_workspace {
 // Fusion works on tiles of 32 x 8 x 8 nodes; the cell view is refreshed
 // tile by tile after fusion.
 constexpr int PF_TX = 32, PF_TY = 8, PF_TZ = 8;
+constexpr int PF_DEPTH_BLOCKS = 64;  // per axis, whatever the image's size
 
 // Per-fusion tile lists (device memory, one slot per tile): the tiles that
-// survive the frustum cull with the camera-frame position of their first
-// node, and the tiles whose cell-view records must be rewritten.
+// survive the culls with the camera-frame position of their first node, which
+// of each tile's rows of nodes changed, and the tiles whose cell-view records
+// must be rewritten with the rows of records concerned.  A tile's rows are
+// bits of a 64-bit word: bit 8 j + k is the row of 32 nodes at (j, k).
 struct FusionList {
     int* count = nullptr;         // [0] fused tiles, [1] tiles to refresh
     int* tile = nullptr;          // fused tile indices
     float4* base = nullptr;       // their first node in the camera frame: x, y, z hi, z lo
     float* step = nullptr;        // 9: camera-frame step per node index along i, j, k
+    float* depth_max = nullptr;   // largest usable depth of each of PF_DEPTH_BLOCKS^2 blocks of the image
+    unsigned long long* rows = nullptr;  // per tile: changed rows (valid where the tile's stamp is the last fusion's)
     int* refresh_tile = nullptr;  // tiles to refresh
+    unsigned long long* refresh_rows = nullptr;  // and their rows
 };
 
 // Where the ray cast can meet the surface: one bit per brick of 8^3 cells,
