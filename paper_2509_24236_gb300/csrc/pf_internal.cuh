@@ -11,6 +11,7 @@
 #include <cmath>
 
 #include "../../include/profusion.h"
+#include "cellpitch.h"
 
 // --------------------------------------------------------------------------
 // TSDF value encoding in the f32 tsdf array.
@@ -176,11 +177,12 @@ struct pf_volume {
     size_t n_nodes = 0;
     void* tsdf = nullptr;      // encoded, see above; float, half or bfloat16 (desc.tsdf_dtype)
     void* weight = nullptr;    // float, or uint8 when desc.weight_u8
-    void* cells = nullptr;     // cell view: 8 values per node (the cell whose lower corner it is)
+    void* cells = nullptr;     // cell view: a record of 8 values per cell, pitched as `pitch` says
     float* cells32 = nullptr;  // 16-/8-bit grids, full view: the same records as floats (x-differences formed)
     int* tile_stamp = nullptr; // per fusion tile: stamp of the last fusion that reached it
     int stamp = 0;             // fusions so far
     int tiles[3] = {0, 0, 0};
+    pf::CellPitch pitch = {0, 0, 0};  // of the records in cells and cells32
     int fitness_variant = 0;
     pf_status last_status = PF_OK;  // last failing status of a call on this volume
     FusionList list;

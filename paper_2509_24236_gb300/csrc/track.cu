@@ -349,6 +349,7 @@ struct FitArgs {
     const void* cells;
     const float* cells32; // 16-/8-bit grids, full view: the records as floats too (else null)
     int nx, ny, nz;
+    int row, plane;       // index strides along y and z of what the launch samples: the node array's, or the cell view's
     double vs;
     double org[3];
     // reduction
@@ -956,7 +957,7 @@ __global__ void __launch_bounds__(32) chunk_build_kernel(FitArgs a, ChunkData* o
     const int kc = min(KC, a.K - k_begin);
     if (SRC != SRC_POSES && a.st->lost) return;  // the fitness launch skips every chunk then
     ChunkData& C = out[blockIdx.x];
-    const int nx = a.nx, nxy = a.nx * a.ny;
+    const int nx = a.row, nxy = a.plane;
     build_particles<SRC, true>(a, k_begin, kc, C.P, C.ref, nullptr);
     __syncwarp();
     const bool mine = t < kc;
@@ -1039,7 +1040,7 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int k_begin = bx * KC;
     const int kc = min(KC, a.K - k_begin);
-    const int nx = a.nx, nxy = a.nx * a.ny;
+    const int nx = a.row, nxy = a.plane;
     const unsigned mx = a.nx - 1, my = a.ny - 1, mz = a.nz - 1;
 
     if (tid == 0) {
@@ -1732,7 +1733,8 @@ void launch_fitness(FitArgs a, int variant, const pf_volume* v, int chunks, cuda
     pf::count_launch();
 }
 
-void fill_volume_args(FitArgs& a, const pf_volume* v)
+// layout: what the launches sample (3: the cell view, else the node array).
+void fill_volume_args(FitArgs& a, const pf_volume* v, int layout)
 {
     a.tsdf = v->tsdf;
     a.weight = v->weight;
@@ -1741,6 +1743,8 @@ void fill_volume_args(FitArgs& a, const pf_volume* v)
     a.nx = v->desc.nx;
     a.ny = v->desc.ny;
     a.nz = v->desc.nz;
+    a.row = layout == 3 ? v->pitch.row : v->desc.nx;
+    a.plane = layout == 3 ? v->pitch.plane : v->desc.nx * v->desc.ny;
     a.vs = v->desc.voxel_size;
     for (int q = 0; q < 3; ++q) a.org[q] = v->desc.origin[q];
 }
@@ -1902,7 +1906,7 @@ static pf_status pf_fitness_impl(const pf_volume* cv, const float* points_dev, i
     a.stride = 1;
     a.K = k;
     a.poses = poses_dev;
-    fill_volume_args(a, v);
+    fill_volume_args(a, v, resolve_fitness_layout(v));
     a.part_S = v->ws.part_S;
     a.part_C = v->ws.part_C;
     a.counter = v->ws.counter;
@@ -1987,7 +1991,7 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
     a.update_mode = p->update_mode;
     a.beta = p->beta;
     a.min_valid_frac = p->min_valid_frac;
-    fill_volume_args(a, v);
+    fill_volume_args(a, v, resolve_fitness_layout(v));
     a.part_S = w.part_S;
     a.part_C = w.part_C;
     a.counter = w.counter;
@@ -2157,7 +2161,7 @@ FitArgs batch_args(const pf_batch* b, int i, SearchState* st, pf_track_stats* st
     a.update_mode = p.update_mode;
     a.beta = p.beta;
     a.min_valid_frac = p.min_valid_frac;
-    fill_volume_args(a, v);
+    fill_volume_args(a, v, b->layout);
     a.part_S = v->ws.part_S;
     a.part_C = v->ws.part_C;
     a.counter = v->ws.counter;
@@ -2663,7 +2667,7 @@ static pf_status pf_fitness_noalloc_impl(const pf_volume* v, const float* points
     a.stride = 1;
     a.K = k;
     a.poses = poses_dev;
-    fill_volume_args(a, v);
+    fill_volume_args(a, v, resolve_fitness_layout(v));
     a.part_S = sc->S;
     a.part_C = sc->C;
     a.counter = &sc->counter;

@@ -382,6 +382,7 @@ struct RefreshArgs {
     void* cells;
     float* cells32;  // 16-/8-bit grids, full view: the float records as well
     int nx, ny, nz;
+    int row, plane;  // pitch of the records
     const int* tile_stamp;
     const int* stamp_dev;
     int all;
@@ -490,6 +491,7 @@ __global__ void __launch_bounds__(TX * TY, 4) cells_refresh_kernel(RefreshArgs a
         if (i >= a.nx - 1 || j >= a.ny - 1) continue;
         const unsigned planes = rows | (rows << 1);  // node planes k0 + dz that the rows touch
         const size_t idx = i + nx * j + nxy * k0;
+        const size_t rec = i + (size_t)a.row * j + (size_t)a.plane * k0;
 #pragma unroll 1
         for (int h = 0; h < TZ; h += HALF) {
             if ((rows >> h & ((1u << HALF) - 1u)) == 0u) continue;
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(TX * TY, 4) cells_refresh_kernel(RefreshArgs a
 #pragma unroll
             for (int dz = 0; dz < HALF; ++dz)
                 if ((rows >> (h + dz) & 1u) && k0 + h + dz < a.nz - 1)
-                    store_record(cells, a.cells32, idx + nxy * (h + dz), v[dz], v[dz + 1]);
+                    store_record(cells, a.cells32, rec + (size_t)a.plane * (h + dz), v[dz], v[dz + 1]);
         }
     }
 }
@@ -533,6 +535,8 @@ pf_status enqueue_refresh(pf_volume* v, cudaStream_t s, int all)
     r.nx = v->desc.nx;
     r.ny = v->desc.ny;
     r.nz = v->desc.nz;
+    r.row = v->pitch.row;
+    r.plane = v->pitch.plane;
     const int n_tiles = v->tiles[0] * v->tiles[1] * v->tiles[2];
     r.tile_stamp = v->tile_stamp;
     r.stamp_dev = v->tile_stamp + n_tiles;
@@ -705,8 +709,10 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     // on points: two or four records per sector) and float records (lanes on
     // particles: no conversions); the narrow view keeps the narrow records
     // only; a float grid has the float records only
-    const size_t bytes32 = vdt == PF_F32 ? 0 : v->n_nodes * 32;
-    const size_t view_bytes = v->n_nodes * 8 * vs;
+    v->pitch = pf::cell_pitch(desc->nx, desc->ny, desc->nz);
+    const size_t n_cells = (size_t)v->pitch.count;
+    const size_t bytes32 = vdt == PF_F32 ? 0 : n_cells * 32;
+    const size_t view_bytes = n_cells * 8 * vs;
     const size_t grid_bytes = v->n_nodes * (ts + ws);
     cudaError_t e = cudaGetDevice(&v->device);
     int mode = desc->cell_view;
@@ -821,8 +827,8 @@ pf_status pf_volume_info(const pf_volume* v, unsigned long long* storage_bytes, 
     const size_t n = v->n_nodes, ts = pf_dtype_size(v->desc.tsdf_dtype), vs = pf_dtype_size(pf_view_dtype(v));
     const size_t n_tiles = (size_t)v->tiles[0] * v->tiles[1] * v->tiles[2];
     size_t b = n * ts + n * (v->desc.weight_u8 ? 1 : 4);
-    if (v->cells) b += n * 8 * vs + sizeof(int) * (n_tiles + 1);
-    if (v->cells32) b += n * 32;
+    if (v->cells) b += (size_t)v->pitch.count * 8 * vs + sizeof(int) * (n_tiles + 1);
+    if (v->cells32) b += (size_t)v->pitch.count * 32;
     if (storage_bytes) *storage_bytes = b;
     if (cell_view) *cell_view = !v->cells ? -1 : (v->cells32 || pf_view_dtype(v) == PF_F32) ? 1 : 2;
     return PF_OK;
