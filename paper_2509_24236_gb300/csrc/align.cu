@@ -29,9 +29,9 @@
 //   * Polish: a damped Gauss-Newton (Levenberg-Marquardt) with its state in
 //     device memory.  gn_kernel accumulates H = sum J^T J (upper triangle),
 //     b = sum J^T r, sum r^2 and the count for the state's candidate pose
-//     (float per thread, FP64 across threads and tiles); gn_step (one thread) reduces the tiles, accepts the candidate if
-//     it lowers the mean squared residual (lambda /= 10) or drops it
-//     (lambda *= 10), solves (H + lambda diag H) d = -b and forms the next
+//     (float per thread, FP64 across threads and tiles); the last block of
+//     the launch accepts the candidate if it lowers the mean squared residual
+//     (lambda /= 10) or drops it (lambda *= 10), solves (H + lambda diag H) d = -b and forms the next
 //     candidate [Exp(d_omega) | d_v] T.  No host round trip: a polish is a
 //     fixed launch sequence.
 #include <algorithm>
@@ -51,12 +51,13 @@ constexpr int RED_THREADS = 256;       // tile reductions
 constexpr float kRound = 12582912.0f;  // 1.5 * 2^23: adding it rounds |v| < 2^22 to an integer
 constexpr int kRoundBits = 0x4B400000;  // its bit pattern
 constexpr int GN_VALS = 29;            // 21 (upper H) + 6 (b) + loss + count
+constexpr int GN_CLASSES = RED_THREADS / GN_VALS;  // 8 classes of tiles, summed apart
 
 struct AlignScratch {
     double* part = nullptr;       // align partials: frames x tiles x 8 (tiles <= AL_TILES)
     size_t part_cap = 0;          // doubles
     long long* acc = nullptr;     // n_nodes fixed-point dL/dV
-    double* gn_part = nullptr;    // AL_TILES x GN_VALS
+    double* gn_part = nullptr;    // (AL_TILES + GN_CLASSES) x GN_VALS
     double* gn_state = nullptr;   // see GnState
     void* frame_pose = nullptr;   // frames x FramePose (the poses prepared once per frame)
     int frame_cap = 0;            // frames
@@ -75,33 +76,13 @@ struct GnState {
     int have_cand;     // a candidate is pending evaluation
     int accepted;
     int step;
-    int pad;
+    // of the running launch: finished blocks of each class, finished classes
+    unsigned class_ticket[GN_CLASSES], ticket;
 };
 
 // ---------------------------------------------------------------------------
 // FP64 helpers
 // ---------------------------------------------------------------------------
-__host__ __device__ inline void so3_exp(const double w[3], double R[9])
-{
-    const double th2 = w[0] * w[0] + w[1] * w[1] + w[2] * w[2];
-    const double th = sqrt(th2);
-    double a, b;
-    if (th < 1e-8) {
-        a = 1.0 - th2 / 6.0;
-        b = 0.5 - th2 / 24.0;
-    } else {
-        a = sin(th) / th;
-        b = (1.0 - cos(th)) / th2;
-    }
-    const double K[9] = {0.0, -w[2], w[1], w[2], 0.0, -w[0], -w[1], w[0], 0.0};
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) {
-            double kk = 0.0;
-            for (int m = 0; m < 3; ++m) kk += K[3 * r + m] * K[3 * m + c];
-            R[3 * r + c] = (r == c ? 1.0 : 0.0) + a * K[3 * r + c] + b * kk;
-        }
-}
-
 // left Jacobian of SO(3): I + (1 - cos th)/th^2 [w]x + (th - sin th)/th^3 [w]x^2
 __device__ inline void so3_left_jacobian(const double w[3], double J[9])
 {
@@ -124,21 +105,6 @@ __device__ inline void so3_left_jacobian(const double w[3], double J[9])
         }
 }
 
-// [Exp(omega) R | Exp(omega) t + v] from a row-major 3x4 (or 4x4) pose
-__device__ inline void perturb(const double* P, const double xi[6], double out[12])
-{
-    double dR[9];
-    so3_exp(xi, dR);
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 4; ++c) {
-            double acc = 0.0;
-            for (int m = 0; m < 3; ++m) acc += dR[3 * r + m] * P[4 * m + c];
-            out[4 * r + c] = acc;
-        }
-        out[4 * r + 3] += xi[3 + r];
-    }
-}
-
 struct GridInfo {
     int nx, ny, nz;
     double inv_vs, org[3];
@@ -155,23 +121,78 @@ struct PoseF {
     int ok;  // the camera lies within 2^21 voxels of the grid
 };
 
-__device__ inline void make_posef(const double T[12], const GridInfo& g, PoseF& P)
+// The pose preparations by the first two warps of a block.  Each is a chain of
+// dependent FP64 operations, a hundred cycles and more apiece, which is
+// microseconds in one thread; every element of a matrix is formed by a thread
+// of its own with the expression one thread would use for it, and the sine and
+// the cosine by the two warps at a time, so the results are the same bits.
+__device__ __forceinline__ void pair_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+
+// T (shared) to a PoseF.
+__device__ inline void pair_make_posef(const double* T, const GridInfo& g, PoseF* out, int* sh_ok)
 {
-    P.ok = 1;
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) {
-            const double A = T[4 * r + c] * g.inv_vs;
-            P.Ahi[3 * r + c] = (float)A;
-            P.Alo[3 * r + c] = (float)(A - (double)P.Ahi[3 * r + c]);
-            P.R[3 * r + c] = (float)T[4 * r + c];
-        }
+    const int tid = threadIdx.x;
+    if (tid == 0) *sh_ok = 1;
+    pair_sync();
+    if (tid < 9) {
+        const int r = tid / 3, c = tid % 3;
+        const double A = T[4 * r + c] * g.inv_vs;
+        const float hi = (float)A;
+        out->Ahi[tid] = hi;
+        out->Alo[tid] = (float)(A - (double)hi);
+        out->R[tid] = (float)T[4 * r + c];
+    } else if (tid >= 32 && tid < 35) {
+        const int r = tid - 32;
         const double tg = (T[4 * r + 3] - g.org[r]) * g.inv_vs;
-        if (!(fabs(tg) < 2097152.0)) P.ok = 0;
-        const double o = P.ok ? floor(tg) : 0.0;
-        P.o[r] = (int)o;
-        P.b[r] = (float)(tg - o);
-        P.t[r] = (float)T[4 * r + 3];
+        const bool ok = fabs(tg) < 2097152.0;
+        if (!ok) *sh_ok = 0;
+        const double o = ok ? floor(tg) : 0.0;
+        out->o[r] = (int)o;
+        out->b[r] = (float)(tg - o);
+        out->t[r] = (float)T[4 * r + 3];
     }
+    pair_sync();
+    if (tid == 0) out->ok = *sh_ok;
+}
+
+// [Exp(omega) R | Exp(omega) t + v] (shared out, 12) from a 3x4 pose P, Exp
+// Rodrigues' formula.  xi: 6 doubles; sh: 16 doubles of shared memory.
+__device__ inline void pair_perturb(const double* P, const double* xi, double* out, double* sh)
+{
+    const int tid = threadIdx.x;
+    const double th2 = xi[0] * xi[0] + xi[1] * xi[1] + xi[2] * xi[2];
+    if (tid == 0 || tid == 32) {
+        const double th = sqrt(th2);
+        if (th < 1e-8)
+            sh[tid >> 5] = tid == 0 ? 1.0 - th2 / 6.0 : 0.5 - th2 / 24.0;
+        else if (tid == 0)
+            sh[0] = sin(th) / th;
+        else
+            sh[1] = (1.0 - cos(th)) / th2;
+    }
+    pair_sync();
+    if (tid < 9) {
+        const int r = tid / 3, c = tid % 3;
+        const double K[9] = {0.0, -xi[2], xi[1], xi[2], 0.0, -xi[0], -xi[1], xi[0], 0.0};
+        double kr[3], kc[3], krc = 0.0;
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {  // (constant indices: the array stays in registers)
+            if (q / 3 == r) kr[q % 3] = K[q];
+            if (q % 3 == c) kc[q / 3] = K[q];
+            if (q == tid) krc = K[q];
+        }
+        double kk = 0.0;
+        for (int m = 0; m < 3; ++m) kk += kr[m] * kc[m];
+        sh[4 + tid] = (r == c ? 1.0 : 0.0) + sh[0] * krc + sh[1] * kk;
+    }
+    pair_sync();
+    if (tid < 12) {
+        const int r = tid / 4, c = tid % 4;
+        double acc = 0.0;
+        for (int m = 0; m < 3; ++m) acc += sh[4 + 3 * r + m] * P[4 * m + c];
+        out[tid] = c == 3 ? acc + xi[3 + r] : acc;
+    }
+    pair_sync();
 }
 
 // One frame of pf_align_loss, prepared once per frame (FP64 work that every
@@ -222,17 +243,31 @@ __device__ inline bool row_split(const float* hi, const float* lo, float x, floa
     return true;
 }
 
+// What a sample reads: the node array, or (records not null) the cell view's
+// 32-byte float records, whose first differences are the ones formed here, so
+// both give the same bits.
+template <typename TS>
+struct Field {
+    const TS* tsdf;
+    const float* records;
+    int row, plane;  // of the records
+};
+
 // Trilinear value t, its gradient in grid units, the cell (linear index of
 // its lower corner) and the fractions of point x under pose P; false when
 // the sample lies in no valid cell (outside the grid, or a node that is
 // unobserved or outside the band -- non-finite in the encoded storage).
-template <typename TS>
-__device__ inline bool sample_f(const TS* tsdf, const GridInfo& g, const PoseF& P, float x, float y, float z,
-                                float& t, float dg[3], long long& base, float f[3])
+// One 256-bit load of a record in place of eight of nodes, or the eight
+// before any test of them, so that they wait together: a test after each was
+// eight waits in a row (4.9 M points' loss 98 -> 63 us, with all derivatives
+// 209 -> 173 us, the scatter's integer reductions being the rest).
+template <typename TS, bool RECORDS>
+__device__ __forceinline__ bool sample_f(const Field<TS>& F, const GridInfo& g, const PoseF& P, float x, float y,
+                                         float z, float& t, float dg[3], int& base, float f[3])
 {
     if (!P.ok || !isfinite(x) || !isfinite(y) || !isfinite(z)) return false;
     const int n[3] = {g.nx, g.ny, g.nz};
-    long long ci[3];
+    int ci[3];
 #pragma unroll
     for (int r = 0; r < 3; ++r) {
         int yi;
@@ -242,27 +277,40 @@ __device__ inline bool sample_f(const TS* tsdf, const GridInfo& g, const PoseF& 
         // floor(u) the same way with round-down (|u| is a few units)
         const float m = __fadd_rd(u, kRound);
         const float fl = __fsub_rn(m, kRound);
-        ci[r] = (long long)P.o[r] + yi + (long long)(__float_as_int(m) - kRoundBits);
+        // (|o| < 2^21, |yi| <= 2^22: no overflow)
+        ci[r] = P.o[r] + yi + (__float_as_int(m) - kRoundBits);
         f[r] = __fsub_rn(u, fl);
-        if (ci[r] < 0 || ci[r] > n[r] - 2) return false;
+        if ((unsigned)ci[r] > (unsigned)(n[r] - 2)) return false;
     }
-    const long long nx = g.nx, nxy = (long long)g.nx * g.ny;
+    const int nx = g.nx, nxy = g.nx * g.ny;
     base = ci[0] + nx * ci[1] + nxy * ci[2];
-    const long long off[8] = {0, 1, nx, nx + 1, nxy, nxy + 1, nxy + nx, nxy + nx + 1};
-    float v[8];
-#pragma unroll
-    for (int c = 0; c < 8; ++c) {
-        v[c] = pf_to_float(tsdf[base + off[c]]);
-        if (!isfinite(v[c])) return false;
+    float v0, v2, v4, v6, dx00, dx10, dx01, dx11;
+    if (RECORDS) {
+        const float* p = F.records + 8 * (size_t)(unsigned)(ci[0] + F.row * ci[1] + F.plane * ci[2]);
+        // (volatile: not to be moved above the range test)
+        asm volatile("ld.global.nc.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+            : "=f"(v0), "=f"(dx00), "=f"(v2), "=f"(dx10), "=f"(v4), "=f"(dx01), "=f"(v6), "=f"(dx11) : "l"(p));
+    } else {
+        const TS* p = F.tsdf + base;
+        const TS e[8] = {p[0], p[1], p[nx], p[nx + 1], p[nxy], p[nxy + 1], p[nxy + nx], p[nxy + nx + 1]};
+        v0 = pf_to_float(e[0]);
+        v2 = pf_to_float(e[2]);
+        v4 = pf_to_float(e[4]);
+        v6 = pf_to_float(e[6]);
+        dx00 = pf_to_float(e[1]) - v0;
+        dx10 = pf_to_float(e[3]) - v2;
+        dx01 = pf_to_float(e[5]) - v4;
+        dx11 = pf_to_float(e[7]) - v6;
     }
-    const float x00 = fmaf(f[0], v[1] - v[0], v[0]);
-    const float x10 = fmaf(f[0], v[3] - v[2], v[2]);
-    const float x01 = fmaf(f[0], v[5] - v[4], v[4]);
-    const float x11 = fmaf(f[0], v[7] - v[6], v[6]);
+    // a difference is finite exactly when both its nodes are
+    if (!(isfinite(dx00) && isfinite(dx10) && isfinite(dx01) && isfinite(dx11))) return false;
+    const float x00 = fmaf(f[0], dx00, v0);
+    const float x10 = fmaf(f[0], dx10, v2);
+    const float x01 = fmaf(f[0], dx01, v4);
+    const float x11 = fmaf(f[0], dx11, v6);
     const float y0 = fmaf(f[1], x10 - x00, x00);
     const float y1 = fmaf(f[1], x11 - x01, x01);
     t = fmaf(f[2], y1 - y0, y0);
-    const float dx00 = v[1] - v[0], dx10 = v[3] - v[2], dx01 = v[5] - v[4], dx11 = v[7] - v[6];
     const float dy0 = fmaf(f[1], dx10 - dx00, dx00), dy1 = fmaf(f[1], dx11 - dx01, dx01);
     dg[0] = fmaf(f[2], dy1 - dy0, dy0);
     dg[1] = fmaf(f[2], (x11 - x01) - (x10 - x00), x10 - x00);
@@ -315,27 +363,16 @@ __device__ __forceinline__ void block_range(int n, long long& beg, long long& en
     end = beg + q + (b < r ? 1 : 0);
 }
 
-// Warps' partial sums (shared sh[warp * NV + i]) to block totals out[i]:
-// thread i adds value i over the warps in order, in FP64.
-template <int NV>
-__device__ inline void warps_to_block(const double* sh, double* out)
-{
-    const int tid = threadIdx.x;
-    if (tid < NV) {
-        double s = 0.0;
-        for (int w = 0; w < AL_THREADS / 32; ++w) s += sh[w * NV + tid];
-        out[tid] = s;
-    }
-    __syncthreads();
-}
-
 // Fixed-order block sum of NV floats per thread, each lane's value carried
 // as an unevaluated float pair (s, c) through the warp's shuffle tree with
 // error-free additions (TwoSum), so the warp sum keeps about twice float
-// precision without the FP64 pipe; warps are then summed in FP64.
-// Block totals in out[0 .. NV) (shared), visible to every thread.
+// precision without the FP64 pipe; thread i then adds value i over the warps
+// in order, in FP64.  The warps' sums go through shared memory as floats and
+// become FP64 in that thread: converting in each warp, on a FP64 pipe that all
+// of them share, made this sum 9 700 cycles of a polish step (29 values), now
+// 3 900.  Block totals in out[0 .. NV) (shared), visible to every thread.
 template <int NV>
-__device__ inline void block_sum_ff(const float* v, double* sh, double* out)
+__device__ inline void block_sum_ff(const float* v, float* sh, double* out)
 {
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     float sv[NV], cv[NV];
@@ -361,25 +398,41 @@ __device__ inline void block_sum_ff(const float* v, double* sh, double* out)
             cv[i] = __fadd_rn(__fadd_rn(ca, cb), err);
         }
     if (lane == 0)
-        for (int i = 0; i < NV; ++i) sh[warp * NV + i] = (double)sv[i] + (double)cv[i];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            sh[2 * (warp * NV + i)] = sv[i];
+            sh[2 * (warp * NV + i) + 1] = cv[i];
+        }
     __syncthreads();
-    warps_to_block<NV>(sh, out);
+    if (tid < NV) {
+        double s = 0.0;
+        for (int w = 0; w < AL_THREADS / 32; ++w)
+            s += (double)sh[2 * (w * NV + tid)] + (double)sh[2 * (w * NV + tid) + 1];
+        out[tid] = s;
+    }
+    __syncthreads();
 }
 
 // Fixed-order block sum of NV floats per thread: the 32 lanes of a warp in
 // float (about one sample per lane in the polish, so float keeps ~1e-6 of
-// the sum), the warps and thread 0's totals in FP64 (out[0 .. NV)).
+// the sum), the warps in FP64 by thread i as above (out[0 .. NV)).
 template <int NV>
-__device__ inline void block_sum_f(float* v, double* sh, double* out)
+__device__ inline void block_sum_f(float* v, float* sh, double* out)
 {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
 #pragma unroll
     for (int i = 0; i < NV; ++i)
         for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(0xffffffffu, v[i], o);
     if (lane == 0)
-        for (int i = 0; i < NV; ++i) sh[warp * NV + i] = (double)v[i];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) sh[warp * NV + i] = v[i];
     __syncthreads();
-    warps_to_block<NV>(sh, out);
+    if (tid < NV) {
+        double s = 0.0;
+        for (int w = 0; w < AL_THREADS / 32; ++w) s += (double)sh[w * NV + tid];
+        out[tid] = s;
+    }
+    __syncthreads();
 }
 
 // ---------------------------------------------------------------------------
@@ -394,34 +447,35 @@ struct AlignArgs {
     const double* poses;  // F x 16
     const double* xi;     // F x 6 or null
     const double* dloss;  // F or null
+    const float* records; // float records of the cell view, or null
+    int row, plane;
     double* part;         // F x tiles x 8
     long long* acc;       // n_nodes or null
     const FramePose* fposes;  // F, from align_prep
 };
 
-// Thread f prepares frame f: its perturbed pose, v and 2 W.
-__global__ void align_prep(const double* poses, const double* xi, const double* dloss, GridInfo g, int F,
-                           FramePose* out)
+// Block f prepares frame f: its perturbed pose, v and 2 W (64 frames: 14.5 us
+// with a thread each in one block, 7.4 us so).
+__global__ void __launch_bounds__(64) align_prep(const double* poses, const double* xi, const double* dloss, GridInfo g,
+                                                 FramePose* out)
 {
-    const int f = blockIdx.x * blockDim.x + threadIdx.x;
-    if (f >= F) return;
-    double x[6] = {0, 0, 0, 0, 0, 0};
-    if (xi)
-        for (int i = 0; i < 6; ++i) x[i] = xi[6 * (size_t)f + i];
-    double T[12];
-    perturb(poses + 16 * (size_t)f, x, T);
-    FramePose fp;
-    make_posef(T, g, fp.P);
-    for (int i = 0; i < 3; ++i) fp.V[i] = (float)x[3 + i];
-    fp.w2 = (float)(2.0 * (dloss ? dloss[f] : 1.0));
-    out[f] = fp;
+    __shared__ double s_xi[6], s_P[12], s_T[12], sh[16];
+    __shared__ int sh_ok;
+    const int f = blockIdx.x, tid = threadIdx.x;
+    if (tid < 6) s_xi[tid] = xi ? xi[6 * (size_t)f + tid] : 0.0;
+    if (tid >= 32 && tid < 44) s_P[tid - 32] = poses[16 * (size_t)f + tid - 32];
+    __syncthreads();
+    pair_perturb(s_P, s_xi, s_T, sh);
+    pair_make_posef(s_T, g, &out[f].P, &sh_ok);
+    if (tid < 3) out[f].V[tid] = (float)s_xi[3 + tid];
+    if (tid == 32) out[f].w2 = (float)(2.0 * (dloss ? dloss[f] : 1.0));
 }
 
-template <typename TS>
+template <typename TS, bool RECORDS>
 __global__ void __launch_bounds__(AL_THREADS) align_kernel(AlignArgs a)
 {
     __shared__ FramePose sF;
-    __shared__ double sh[(AL_THREADS / 32) * 8];
+    __shared__ float sh[(AL_THREADS / 32) * 8 * 2];
     const int f = blockIdx.y, tid = threadIdx.x;
     block_copy_words(a.fposes + f, &sF);
     const PoseF& sP = sF.P;
@@ -429,17 +483,21 @@ __global__ void __launch_bounds__(AL_THREADS) align_kernel(AlignArgs a)
     const int n = a.counts ? min(a.counts[f], a.n_max) : a.n_max;
     long long beg, end;
     block_range(n, beg, end);
-    const TS* tsdf = static_cast<const TS*>(a.tsdf);
+    const Field<TS> field = {static_cast<const TS*>(a.tsdf), a.records, a.row, a.plane};
     const float inv_vs = (float)a.g.inv_vs;
     // dL/dV increments in units of 2^-40: round(2 W t w 2^40), formed in
     // float (exact for W = 1, one float rounding otherwise)
     const float w2 = sF.w2;
     float acc[8] = {0, 0, 0, 0, 0, 0, 0, 0};  // L, C, gw[3], gv[3]
+    const float4* pts = a.pts + (size_t)f * a.n_max;
+    float4 next = beg + tid < end ? __ldg(pts + beg + tid) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
     for (long long e = beg + tid; e < end; e += AL_THREADS) {
-        const float4 p = __ldg(a.pts + (size_t)f * a.n_max + e);
+        // (the next point is on its way while this one's record is)
+        const float4 p = next;
+        if (e + AL_THREADS < end) next = __ldg(pts + e + AL_THREADS);
         float t, dg[3], fr[3];
-        long long base;
-        if (!sample_f(tsdf, a.g, sP, p.x, p.y, p.z, t, dg, base, fr)) continue;
+        int base;
+        if (!sample_f<TS, RECORDS>(field, a.g, sP, p.x, p.y, p.z, t, dg, base, fr)) continue;
         float q[3];
         transform_f(sP, p.x, p.y, p.z, q);
         const float gt[3] = {dg[0] * inv_vs, dg[1] * inv_vs, dg[2] * inv_vs};
@@ -454,12 +512,12 @@ __global__ void __launch_bounds__(AL_THREADS) align_kernel(AlignArgs a)
         acc[6] = fmaf(t2, gt[1], acc[6]);
         acc[7] = fmaf(t2, gt[2], acc[7]);
         if (a.acc) {
-            const long long nx = a.g.nx, nxy = (long long)a.g.nx * a.g.ny;
+            const int nx = a.g.nx, nxy = a.g.nx * a.g.ny;
 #pragma unroll
             for (int c = 0; c < 8; ++c) {
                 const float w = ((c & 1) ? fr[0] : 1.0f - fr[0]) * (((c >> 1) & 1) ? fr[1] : 1.0f - fr[1]) *
                                 (((c >> 2) & 1) ? fr[2] : 1.0f - fr[2]);
-                const long long idx = base + ((c & 1) ? 1 : 0) + (((c >> 1) & 1) ? nx : 0) + (((c >> 2) & 1) ? nxy : 0);
+                const int idx = base + ((c & 1) ? 1 : 0) + (((c >> 1) & 1) ? nx : 0) + (((c >> 2) & 1) ? nxy : 0);
                 const long long inc = fix40(w2 * (t * w));
                 if (inc != 0) atomicAdd(reinterpret_cast<unsigned long long*>(a.acc + idx), (unsigned long long)inc);
             }
@@ -481,7 +539,8 @@ __device__ inline void tile_sum(const double* part, int tiles, double* sh, doubl
     const int tid = threadIdx.x, i = tid % NV, j = tid / NV;
     if (j < J) {
         double acc = 0.0;
-        for (int y = j; y < tiles; y += J) acc += part[(size_t)y * NV + i];
+#pragma unroll 4
+        for (int y = j; y < tiles; y += J) acc += __ldcg(part + (size_t)y * NV + i);
         sh[j * NV + i] = acc;
     }
     __syncthreads();
@@ -544,10 +603,33 @@ __device__ __forceinline__ float fixed40_to_float(long long v)
     return __uint_as_float((v < 0 ? 0x80000000u : 0u) | ((unsigned)(e + 127) << 23) | ((unsigned)q & 0x7fffffu));
 }
 
-__global__ void fixed_to_float(const long long* acc, float* out, size_t n)
+// The accumulator to floats, and back to zero where it was not, so that the
+// next call finds it zero (a separate fill wrote 8 bytes a node more).  Bound
+// by HBM: 8 bytes read and 4 written a node.  Four nodes a thread at a time
+// when the output is 16-byte aligned, else one.
+template <bool QUADS>
+__global__ void __launch_bounds__(256) fixed_to_float(long long* acc, float* out, size_t n)
 {
-    for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-        out[i] = fixed40_to_float(acc[i]);
+    const size_t first = blockIdx.x * (size_t)blockDim.x + threadIdx.x, step = (size_t)gridDim.x * blockDim.x;
+    size_t done = 0;
+    if constexpr (QUADS) {
+        longlong2* acc2 = reinterpret_cast<longlong2*>(acc);
+        for (size_t i = first; i < n / 4; i += step) {
+            const longlong2 a = __ldcs(acc2 + 2 * i), b = __ldcs(acc2 + 2 * i + 1);
+            reinterpret_cast<float4*>(out)[i] = make_float4(fixed40_to_float(a.x), fixed40_to_float(a.y),
+                                                            fixed40_to_float(b.x), fixed40_to_float(b.y));
+            if ((a.x | a.y | b.x | b.y) != 0) {
+                acc2[2 * i] = make_longlong2(0, 0);
+                acc2[2 * i + 1] = make_longlong2(0, 0);
+            }
+        }
+        done = n / 4 * 4;
+    }
+    for (size_t i = done + first; i < n; i += step) {
+        const long long v = acc[i];
+        out[i] = fixed40_to_float(v);
+        if (v != 0) acc[i] = 0;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -556,159 +638,277 @@ __global__ void fixed_to_float(const long long* acc, float* out, size_t n)
 struct GnArgs {
     const void* tsdf;
     GridInfo g;
+    const float* records;  // float records of the cell view, or null
+    int row, plane;
     const float4* pts;
     const int* n_dev;
     int n_max;
     GnState* st;
-    double* part;      // tiles x GN_VALS
-    const PoseF* pc;   // the candidate prepared by gn_begin / gn_step
+    double* part;      // (tiles + GN_CLASSES) x GN_VALS
+    PoseF* pc;         // the candidate prepared by gn_begin or the step before
+    // the step at the end of the launch
+    int mode;          // 0: take the evaluated input pose; 1: accept or drop the candidate
+    double* pose_out;  // or null: not the last step
+    double* trace;     // or null
+    int* accepted_out; // or null
 };
 
-template <typename TS>
-__global__ void __launch_bounds__(AL_THREADS) gn_kernel(GnArgs a)
+// The 6x6 system A d = y by Gaussian elimination with partial pivoting, by the
+// first warp: A | y in shared memory as 6 rows of 7, each element eliminated
+// by a lane of its own with the operations of the serial loop, in its order
+// (so a column costs one division and two more FP64 instructions; magnitudes
+// are compared as integers).  False (in each lane) when a pivot column is zero
+// or not a number.
+__device__ inline bool warp_solve6(double (*A)[7], double* d)
 {
-    __shared__ PoseF sP;
-    __shared__ double sh[(AL_THREADS / 32) * GN_VALS];
-    const int tid = threadIdx.x;
-    if (!a.st->have_cand) return;  // no candidate this step: gn_step ignores the partials
-    block_copy_words(a.pc, &sP);
-    const int n = a.n_dev ? min(*a.n_dev, a.n_max) : a.n_max;
-    long long beg, end;
-    block_range(n, beg, end);
-    const TS* tsdf = static_cast<const TS*>(a.tsdf);
-    const float inv_vs = (float)a.g.inv_vs;
-    float acc[GN_VALS];
+    const int lane = threadIdx.x;
+    auto magnitude = [](double x) { return __double_as_longlong(x) & 0x7fffffffffffffffll; };
+    const long long inf = 0x7ff0000000000000ll;
 #pragma unroll
-    for (int i = 0; i < GN_VALS; ++i) acc[i] = 0.0f;
-    for (long long e = beg + tid; e < end; e += AL_THREADS) {
-        const float4 p = __ldg(a.pts + e);
-        float t, dg[3], fr[3];
-        long long base;
-        if (!sample_f(tsdf, a.g, sP, p.x, p.y, p.z, t, dg, base, fr)) continue;
-        float q[3];
-        transform_f(sP, p.x, p.y, p.z, q);
-        const float gt[3] = {dg[0] * inv_vs, dg[1] * inv_vs, dg[2] * inv_vs};
-        const float J[6] = {q[1] * gt[2] - q[2] * gt[1], q[2] * gt[0] - q[0] * gt[2], q[0] * gt[1] - q[1] * gt[0],
-                            gt[0], gt[1], gt[2]};
-        int m = 0;
-#pragma unroll
-        for (int r = 0; r < 6; ++r)
-#pragma unroll
-            for (int c = r; c < 6; ++c) {
-                acc[m] = fmaf(J[r], J[c], acc[m]);
-                ++m;
-            }
-#pragma unroll
-        for (int r = 0; r < 6; ++r) acc[21 + r] = fmaf(J[r], t, acc[21 + r]);
-        acc[27] = fmaf(t, t, acc[27]);
-        acc[28] += 1.0f;
-    }
-    __shared__ double tot[GN_VALS];
-    block_sum_f<GN_VALS>(acc, sh, tot);
-    if (tid < GN_VALS) a.part[(size_t)blockIdx.x * GN_VALS + tid] = tot[tid];
-}
-
-// solve the 6x6 system A d = y by Gaussian elimination with partial pivoting
-__device__ inline bool solve6(double* A, double* y, double d[6])
-{
     for (int col = 0; col < 6; ++col) {
         int piv = col;
-        for (int r = col + 1; r < 6; ++r)
-            if (fabs(A[6 * r + col]) > fabs(A[6 * piv + col])) piv = r;
-        if (!(fabs(A[6 * piv + col]) > 0.0)) return false;
-        if (piv != col) {
-            for (int c = 0; c < 6; ++c) {
-                const double tmp = A[6 * col + c];
-                A[6 * col + c] = A[6 * piv + c];
-                A[6 * piv + c] = tmp;
+        long long big = magnitude(A[col][col]);
+        for (int q = col + 1; q < 6; ++q) {
+            const long long v = magnitude(A[q][col]);
+            if (v <= inf && big <= inf && v > big) {
+                piv = q;
+                big = v;
             }
-            const double tmp = y[col];
-            y[col] = y[piv];
-            y[piv] = tmp;
         }
-        for (int r = col + 1; r < 6; ++r) {
-            const double m = A[6 * r + col] / A[6 * col + col];
-            for (int c = col; c < 6; ++c) A[6 * r + c] -= m * A[6 * col + c];
-            y[r] -= m * y[col];
+        if (big == 0 || big > inf) return false;
+        // exchange rows col and piv
+        double x = 0.0, y = 0.0;
+        if (lane < 7) {
+            x = A[piv][lane];
+            y = A[col][lane];
         }
+        __syncwarp();
+        if (lane < 7) {
+            A[piv][lane] = y;
+            A[col][lane] = x;
+        }
+        __syncwarp();
+        const int w = 6 - col, r = col + 1 + lane / w, c = col + 1 + lane % w;  // 30 elements at most
+        if (r < 6) {
+            const double m = A[r][col] / A[col][col];
+            A[r][c] = A[r][c] - m * A[col][c];  // (column col is not written)
+        }
+        __syncwarp();
     }
-    for (int r = 5; r >= 0; --r) {
-        double acc = y[r];
-        for (int c = r + 1; c < 6; ++c) acc -= A[6 * r + c] * d[c];
-        d[r] = acc / A[6 * r + r];
+    // back substitution: the products with a new unknown by a lane per row,
+    // each row's subtractions in their order
+    double prod[6] = {0, 0, 0, 0, 0, 0};  // lane r: A[r][c] d[c]
+    const int row = lane < 6 ? lane : 5;
+#pragma unroll
+    for (int q = 5; q >= 0; --q) {
+        double acc = A[row][6];
+#pragma unroll
+        for (int k = q + 1; k < 6; ++k) acc -= prod[k];
+        const double x = __shfl_sync(0xffffffffu, acc / A[row][row], q);
+        prod[q] = A[row][q] * x;
+        if (lane == q) d[q] = x;
     }
+    __syncwarp();
     return true;
 }
 
-// The input pose becomes the first candidate to evaluate.
-__global__ void gn_begin(GnState* st, const double* pose_in, GridInfo g, PoseF* pc)
+// Shared memory of the step.
+struct GnShared {
+    double s[GN_VALS];
+    double A[6][7];
+    double d[6], T[12], Tc[12], rot[16];
+    double obj, lambda;
+    int take, ok, solved;
+};
+
+// One step by the block's first two warps, after the candidate's sums (sh.s):
+// mode 0 takes the evaluated input pose as the current one, mode 1 accepts or
+// drops the evaluated candidate; then the next candidate is formed.
+__device__ inline void gn_step(const GnArgs& a, bool evaluated, GnShared& sh)
 {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    for (int i = 0; i < 12; ++i) st->Tc[i] = pose_in[i];
-    make_posef(st->Tc, g, *pc);
+    const int tid = threadIdx.x;
+    GnState* st = a.st;
+    if (tid == 0) {
+        double obj = st->obj, lambda = st->lambda;
+        int take = 0, accepted = st->accepted;
+        if (evaluated) {
+            const double objc = sh.s[28] > 0.0 ? sh.s[27] / sh.s[28] : INFINITY;
+            take = a.mode == 0 || objc < obj;
+            if (take) obj = objc;
+            if (a.mode == 1) {
+                lambda = take ? lambda / 10.0 : lambda * 10.0;
+                accepted += take;
+            } else if (!take) {
+                lambda *= 10.0;
+            }
+        }
+        const int step = st->step + (a.mode == 1 ? 1 : 0);
+        st->obj = sh.obj = obj;
+        st->lambda = sh.lambda = lambda;
+        st->accepted = accepted;
+        st->step = step;
+        st->have_cand = 0;
+        sh.take = take;
+        if (a.trace) a.trace[step] = obj;
+        if (a.accepted_out) *a.accepted_out = accepted;
+    }
+    pair_sync();
+    // the accepted pose and its system, kept in the state
+    const bool take = sh.take != 0;
+    if (tid < 12) {
+        sh.T[tid] = take ? st->Tc[tid] : st->T[tid];
+        st->T[tid] = sh.T[tid];
+    }
+    if (tid < 42) {
+        const int r = tid / 7, c = tid % 7, lo = min(r, c), hi = max(r, c);
+        double v;
+        if (c == 6) {
+            v = take ? sh.s[21 + r] : st->b[r];
+            st->b[r] = v;
+            v = -v;
+        } else {
+            v = take ? sh.s[lo * 6 - lo * (lo - 1) / 2 + hi - lo] : st->H[6 * r + c];
+            st->H[6 * r + c] = v;
+            if (r == c) v += sh.lambda * v;
+        }
+        sh.A[r][c] = v;
+    }
+    pair_sync();
+    if (a.pose_out && tid < 16) a.pose_out[tid] = tid < 12 ? sh.T[tid] : tid == 15 ? 1.0 : 0.0;
+    // next candidate
+    if (!(sh.obj < INFINITY)) return;
+    if (tid < 32) {
+        const bool solved = warp_solve6(sh.A, sh.d);
+        if (tid == 0) sh.solved = solved;
+    }
+    pair_sync();
+    if (!sh.solved) return;
+    pair_perturb(sh.T, sh.d, sh.Tc, sh.rot);
+    if (tid < 12) st->Tc[tid] = sh.Tc[tid];
+    pair_make_posef(sh.Tc, a.g, a.pc, &sh.ok);
+    if (tid == 0) st->have_cand = 1;
+}
+
+// Sums of H, b, the squared residuals and the count over the block's points
+// for the candidate.  The blocks' sums are added by classes (tile y is of class
+// y mod 8), each by the last block of the class to finish, and the last class
+// to finish adds the classes and makes the step (ticket counters, no
+// spinning): a step is one launch.  Bound by the latency of its parts: a point
+// a thread, a gather and the sums about 13 000 cycles, then the step's chain of
+// FP64 operations about 20 000, twelve of them the 6x6 solve.  320x240 points,
+// ten steps: 497 -> 271 us (a step was two launches, the second one thread's
+// work of 35 us).
+template <typename TS, bool RECORDS>
+__global__ void __launch_bounds__(AL_THREADS) gn_kernel(GnArgs a)
+{
+    __shared__ PoseF sP;
+    __shared__ float sh[(AL_THREADS / 32) * GN_VALS];
+    __shared__ GnShared step;
+    __shared__ int s_last;
+    const int tid = threadIdx.x;
+    if (a.st->have_cand) {  // (else the step ignores the partials)
+        block_copy_words(static_cast<const PoseF*>(a.pc), &sP);
+        const int n = a.n_dev ? min(*a.n_dev, a.n_max) : a.n_max;
+        long long beg, end;
+        block_range(n, beg, end);
+        const Field<TS> field = {static_cast<const TS*>(a.tsdf), a.records, a.row, a.plane};
+        const float inv_vs = (float)a.g.inv_vs;
+        float acc[GN_VALS];
+#pragma unroll
+        for (int i = 0; i < GN_VALS; ++i) acc[i] = 0.0f;
+        for (long long e = beg + tid; e < end; e += AL_THREADS) {
+            const float4 p = __ldg(a.pts + e);
+            float t, dg[3], fr[3];
+            int base;
+            if (!sample_f<TS, RECORDS>(field, a.g, sP, p.x, p.y, p.z, t, dg, base, fr)) continue;
+            float q[3];
+            transform_f(sP, p.x, p.y, p.z, q);
+            const float gt[3] = {dg[0] * inv_vs, dg[1] * inv_vs, dg[2] * inv_vs};
+            const float J[6] = {q[1] * gt[2] - q[2] * gt[1], q[2] * gt[0] - q[0] * gt[2], q[0] * gt[1] - q[1] * gt[0],
+                                gt[0], gt[1], gt[2]};
+            int m = 0;
+#pragma unroll
+            for (int r = 0; r < 6; ++r)
+#pragma unroll
+                for (int c = r; c < 6; ++c) {
+                    acc[m] = fmaf(J[r], J[c], acc[m]);
+                    ++m;
+                }
+#pragma unroll
+            for (int r = 0; r < 6; ++r) acc[21 + r] = fmaf(J[r], t, acc[21 + r]);
+            acc[27] = fmaf(t, t, acc[27]);
+            acc[28] += 1.0f;
+        }
+        __shared__ double tot[GN_VALS];
+        block_sum_f<GN_VALS>(acc, sh, tot);
+        if (tid < GN_VALS) a.part[(size_t)blockIdx.x * GN_VALS + tid] = tot[tid];
+    }
+    __threadfence();
+    __syncthreads();
+    const int tiles = gridDim.x, cls = blockIdx.x % GN_CLASSES;
+    if (tid == 0) {
+        const unsigned members = (unsigned)((tiles - cls + GN_CLASSES - 1) / GN_CLASSES);
+        s_last = atomicAdd(&a.st->class_ticket[cls], 1u) == members - 1;
+    }
+    __syncthreads();
+    if (!s_last || tid >= 64) return;
+    __threadfence();
+    double* sums = a.part + (size_t)tiles * GN_VALS;
+    const bool evaluated = a.st->have_cand != 0;
+    if (evaluated && tid < GN_VALS) {
+        // loads 13 at a time (37 tiles in a class): one by one each addition
+        // waits for L2
+        double s = 0.0;
+        for (int y0 = cls; y0 < tiles; y0 += 13 * GN_CLASSES) {
+            double v[13];
+#pragma unroll
+            for (int q = 0; q < 13; ++q) {
+                const int y = y0 + q * GN_CLASSES;
+                v[q] = __ldcg(a.part + (size_t)min(y, tiles - 1) * GN_VALS + tid);
+            }
+#pragma unroll
+            for (int q = 0; q < 13; ++q)
+                if (y0 + q * GN_CLASSES < tiles) s += v[q];
+        }
+        sums[cls * GN_VALS + tid] = s;
+        __threadfence();
+    }
+    pair_sync();
+    if (tid == 0) {
+        a.st->class_ticket[cls] = 0u;
+        s_last = atomicAdd(&a.st->ticket, 1u) == (unsigned)min(tiles, GN_CLASSES) - 1;
+    }
+    pair_sync();
+    if (!s_last) return;
+    __threadfence();
+    if (evaluated && tid < GN_VALS) {
+        double s = 0.0;
+#pragma unroll
+        for (int q = 0; q < GN_CLASSES; ++q) s += __ldcg(sums + q * GN_VALS + tid);
+        step.s[tid] = s;
+    }
+    pair_sync();
+    if (tid == 0) a.st->ticket = 0u;
+    gn_step(a, evaluated, step);
+}
+
+// The input pose becomes the first candidate to evaluate.
+__global__ void __launch_bounds__(64) gn_begin(GnState* st, const double* pose_in, GridInfo g, PoseF* pc)
+{
+    __shared__ double T[12];
+    __shared__ int sh_ok;
+    const int tid = threadIdx.x;
+    if (tid < 12) st->Tc[tid] = T[tid] = pose_in[tid];
+    __syncthreads();
+    pair_make_posef(T, g, pc, &sh_ok);
+    if (tid != 0) return;
     st->lambda = 1e-3;
     st->accepted = 0;
     st->step = 0;
     st->obj = INFINITY;
     st->have_cand = 1;
-}
-
-// mode 0: take the evaluated input pose as the current one; mode 1: one
-// step (accept or drop the evaluated candidate).  Then form the next
-// candidate.
-__global__ void __launch_bounds__(RED_THREADS) gn_step(GnState* st, const double* part, int tiles, int mode,
-                                                       double* pose_out, double* trace, int* accepted_out,
-                                                       GridInfo g, PoseF* pc)
-{
-    __shared__ double sh[RED_THREADS];
-    __shared__ double s[GN_VALS];
-    const bool evaluated = st->have_cand != 0;
-    if (evaluated) tile_sum<GN_VALS>(part, tiles, sh, s);
-    if (threadIdx.x != 0) return;
-    if (evaluated) {
-        const double objc = s[28] > 0.0 ? s[27] / s[28] : INFINITY;
-        if (mode == 0 || objc < st->obj) {
-            for (int i = 0; i < 12; ++i) st->T[i] = st->Tc[i];
-            int m = 0;
-            for (int r = 0; r < 6; ++r)
-                for (int c = r; c < 6; ++c) {
-                    st->H[6 * r + c] = s[m];
-                    st->H[6 * c + r] = s[m];
-                    ++m;
-                }
-            for (int r = 0; r < 6; ++r) st->b[r] = s[21 + r];
-            st->obj = objc;
-            if (mode == 1) {
-                st->lambda /= 10.0;
-                st->accepted += 1;
-            }
-        } else {
-            st->lambda *= 10.0;
-        }
-    }
-    if (mode == 1) st->step += 1;
-    if (trace) trace[st->step] = st->obj;
-    // next candidate
-    st->have_cand = 0;
-    if (st->obj < INFINITY) {
-        double A[36], y[6], d[6];
-        for (int i = 0; i < 36; ++i) A[i] = st->H[i];
-        for (int r = 0; r < 6; ++r) {
-            A[7 * r] += st->lambda * st->H[7 * r];
-            y[r] = -st->b[r];
-        }
-        if (solve6(A, y, d)) {
-            perturb(st->T, d, st->Tc);
-            make_posef(st->Tc, g, *pc);
-            st->have_cand = 1;
-        }
-    }
-    if (pose_out) {
-        for (int i = 0; i < 12; ++i) pose_out[i] = st->T[i];
-        pose_out[12] = pose_out[13] = pose_out[14] = 0.0;
-        pose_out[15] = 1.0;
-    }
-    if (accepted_out) *accepted_out = st->accepted;
+    for (int q = 0; q < GN_CLASSES; ++q) st->class_ticket[q] = 0u;
+    st->ticket = 0u;
 }
 
 GridInfo grid_info(const pf_volume* v)
@@ -722,25 +922,44 @@ GridInfo grid_info(const pf_volume* v)
     return g;
 }
 
-template <template <typename> class K, typename Args>
-void launch_storage(const pf_volume* v, dim3 grid, cudaStream_t s, const Args& a)
+// Float records of the volume's own stored values, which samples can read in
+// place of its nodes: a float grid's view, or a narrow grid's full view (not a
+// float grid's narrower search view, which holds rounded values).
+const float* float_records(const pf_volume* v)
 {
+    if (pf_view_dtype(v) != v->desc.tsdf_dtype) return nullptr;
+    return v->desc.tsdf_dtype == PF_F32 ? static_cast<const float*>(v->cells) : v->cells32;
+}
+
+template <template <typename, bool> class K, typename Args>
+void launch_storage(const pf_volume* v, dim3 grid, cudaStream_t s, Args& a)
+{
+    a.records = float_records(v);
+    a.row = v->pitch.row;
+    a.plane = v->pitch.plane;
+    if (a.records) {  // (the storage type of the nodes does not matter)
+        K<float, true>::run(grid, s, a);
+        return;
+    }
     switch (v->desc.tsdf_dtype) {
-    case PF_F16: K<__half>::run(grid, s, a); break;
-    case PF_BF16: K<__nv_bfloat16>::run(grid, s, a); break;
-    case PF_FP8E4M3: K<__nv_fp8_e4m3>::run(grid, s, a); break;
-    default: K<float>::run(grid, s, a); break;
+    case PF_F16: K<__half, false>::run(grid, s, a); break;
+    case PF_BF16: K<__nv_bfloat16, false>::run(grid, s, a); break;
+    case PF_FP8E4M3: K<__nv_fp8_e4m3, false>::run(grid, s, a); break;
+    default: K<float, false>::run(grid, s, a); break;
     }
 }
 
-template <typename TS>
+template <typename TS, bool RECORDS>
 struct AlignLaunch {
-    static void run(dim3 grid, cudaStream_t s, const AlignArgs& a) { align_kernel<TS><<<grid, AL_THREADS, 0, s>>>(a); }
+    static void run(dim3 grid, cudaStream_t s, const AlignArgs& a)
+    {
+        align_kernel<TS, RECORDS><<<grid, AL_THREADS, 0, s>>>(a);
+    }
 };
 
-template <typename TS>
+template <typename TS, bool RECORDS>
 struct GnLaunch {
-    static void run(dim3 grid, cudaStream_t s, const GnArgs& a) { gn_kernel<TS><<<grid, AL_THREADS, 0, s>>>(a); }
+    static void run(dim3 grid, cudaStream_t s, const GnArgs& a) { gn_kernel<TS, RECORDS><<<grid, AL_THREADS, 0, s>>>(a); }
 };
 
 AlignScratch& scratch_of(const pf_volume* v)
@@ -796,8 +1015,17 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
         PF_CUDA(pf::dev_malloc(&sc.frame_pose, (size_t)n_frames * sizeof(FramePose)));
         sc.frame_cap = n_frames;
     }
-    if (grad_tsdf_dev && !sc.acc) PF_CUDA(pf::dev_malloc(&sc.acc, v->n_nodes * sizeof(long long)));
-    if (grad_tsdf_dev) PF_CUDA(cudaMemsetAsync(sc.acc, 0, v->n_nodes * sizeof(long long), s));
+    // the accumulator is zero between calls: fixed_to_float leaves it so
+    if (grad_tsdf_dev && !sc.acc) {
+        long long* acc = nullptr;
+        PF_CUDA(pf::dev_malloc(&acc, v->n_nodes * sizeof(long long)));
+        const cudaError_t e = cudaMemsetAsync(acc, 0, v->n_nodes * sizeof(long long), s);
+        if (e != cudaSuccess) {
+            cudaFree(acc);
+            return pf::cuda_status(e);
+        }
+        sc.acc = acc;
+    }
     AlignArgs a;
     a.tsdf = v->tsdf;
     a.g = grid_info(v);
@@ -810,21 +1038,24 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
     a.part = sc.part;
     a.acc = grad_tsdf_dev ? sc.acc : nullptr;
     a.fposes = static_cast<const FramePose*>(sc.frame_pose);
-    align_prep<<<(n_frames + 63) / 64, 64, 0, s>>>(poses_dev, xi_dev, dloss_dev, a.g, n_frames,
-                                                   static_cast<FramePose*>(sc.frame_pose));
+    align_prep<<<n_frames, 64, 0, s>>>(poses_dev, xi_dev, dloss_dev, a.g, static_cast<FramePose*>(sc.frame_pose));
     launch_storage<AlignLaunch>(v, dim3(tiles, n_frames), s, a);
-    pf::count_launch(2);
-    PF_LAUNCHED();
     align_finish<<<n_frames, RED_THREADS, 0, s>>>(sc.part, tiles, xi_dev, dloss_dev, loss_dev, count_dev,
                                                   grad_xi_dev);
-    pf::count_launch();
-    PF_LAUNCHED();
+    pf::count_launch(3);
     if (grad_tsdf_dev) {
-        fixed_to_float<<<4 * 152, 256, 0, s>>>(sc.acc, grad_tsdf_dev, v->n_nodes);
+        if (((uintptr_t)grad_tsdf_dev & 15) == 0)
+            fixed_to_float<true><<<8 * 152, 256, 0, s>>>(sc.acc, grad_tsdf_dev, v->n_nodes);
+        else
+            fixed_to_float<false><<<8 * 152, 256, 0, s>>>(sc.acc, grad_tsdf_dev, v->n_nodes);
         pf::count_launch();
-        PF_LAUNCHED();
     }
-    return PF_OK;
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess && grad_tsdf_dev) {  // the accumulator may not be zero: a new one for the next call
+        cudaFree(sc.acc);
+        sc.acc = nullptr;
+    }
+    return pf::cuda_status(e);
 }
 
 static pf_status pf_polish_impl(const pf_volume* v, const float* points_dev, const int* n_dev, int n_max,
@@ -835,7 +1066,7 @@ static pf_status pf_polish_impl(const pf_volume* v, const float* points_dev, con
     if (((uintptr_t)points_dev & 15) != 0) return PF_ERR_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     AlignScratch& sc = scratch_of(v);
-    if (!sc.gn_part) PF_CUDA(pf::dev_malloc(&sc.gn_part, (size_t)AL_TILES * GN_VALS * sizeof(double)));
+    if (!sc.gn_part) PF_CUDA(pf::dev_malloc(&sc.gn_part, (size_t)(AL_TILES + GN_CLASSES) * GN_VALS * sizeof(double)));
     if (!sc.gn_state) PF_CUDA(pf::dev_malloc(&sc.gn_state, sizeof(GnState)));
     if (!sc.gn_pose) PF_CUDA(pf::dev_malloc(&sc.gn_pose, sizeof(PoseF)));
     PoseF* pc = static_cast<PoseF*>(sc.gn_pose);
@@ -851,17 +1082,15 @@ static pf_status pf_polish_impl(const pf_volume* v, const float* points_dev, con
     a.part = sc.gn_part;
     a.pc = pc;
     // evaluate the input pose, then `steps` candidates
-    gn_begin<<<1, 1, 0, s>>>(st, pose_dev, a.g, pc);
-    launch_storage<GnLaunch>(v, dim3(AL_TILES), s, a);
-    gn_step<<<1, RED_THREADS, 0, s>>>(st, sc.gn_part, AL_TILES, 0, steps == 0 ? pose_dev : nullptr, trace_dev,
-                                      accepted_dev, a.g, pc);
-    pf::count_launch(3);
-    PF_LAUNCHED();
-    for (int k = 0; k < steps; ++k) {
+    a.trace = trace_dev;
+    a.accepted_out = accepted_dev;
+    gn_begin<<<1, 64, 0, s>>>(st, pose_dev, a.g, pc);
+    pf::count_launch();
+    for (int k = 0; k <= steps; ++k) {
+        a.mode = k == 0 ? 0 : 1;
+        a.pose_out = k == steps ? pose_dev : nullptr;
         launch_storage<GnLaunch>(v, dim3(AL_TILES), s, a);
-        gn_step<<<1, RED_THREADS, 0, s>>>(st, sc.gn_part, AL_TILES, 1, k == steps - 1 ? pose_dev : nullptr,
-                                          trace_dev, accepted_dev, a.g, pc);
-        pf::count_launch(2);
+        pf::count_launch();
         PF_LAUNCHED();
     }
     return PF_OK;
