@@ -127,6 +127,7 @@ struct pf_workspace {
     unsigned int* chunk_counter = nullptr;  // per chunk: tickets of its point tiles (zeroed, reset by the last)
     float* chunk_E = nullptr;        // per particle: fitness of the search iteration (chunk_cap x 32)
     int* chunk_C = nullptr;          // per particle: valid points
+    void* select = nullptr;          // partial results of the selection, see track.cu
     // decimated point sets in a locality order (see track.cu): each point's
     // tile, the reordered kept points of up to three strides, counters
     int* point_tile = nullptr;       // pix_cap

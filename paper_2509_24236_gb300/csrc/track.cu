@@ -58,6 +58,7 @@ struct SearchState {
     double P[12];     // current pose, row-major 3x4 camera-to-world
     double P0[12];    // initial pose
     double s[2];      // search size (deg, cm) of the current iteration
+    double w[2];      // the same in radians and metres
     int lost;         // frame declared lost
     int pending_s;    // mean update: s waits for E(P_new)
     int n_points;
@@ -323,6 +324,16 @@ constexpr int SUBTILE = FIT_THREADS * PPT;
 
 enum Source { SRC_POSES = 0, SRC_SEARCH = 1, SRC_EVAL = 2 };
 
+// What the blocks of search_select_kernel leave for its last one.
+constexpr int SEL_CLASSES = 8;  // classes of particles: 32 consecutive ones of every 256
+struct SelectPart {
+    double sum[SEL_CLASSES][6];  // of the advantage set's templates
+    float e[SEL_CLASSES];        // smallest fitness
+    int k[SEL_CLASSES];          // of the lowest such particle
+    int n_adv[SEL_CLASSES];
+    unsigned ticket;             // finished blocks (zero between launches)
+};
+
 struct FitArgs {
     const float4* pts;
     const int* n_dev;     // device point count, or nullptr to use n_host
@@ -333,12 +344,13 @@ struct FitArgs {
     float pm_threshold;   // particles on lanes when the chunk's spread (voxels) is below this
     const float* templ;   // SRC_SEARCH: templates, row k = particle k
     const void* chunks;   // the launch's particle chunks built by chunk_build_kernel, or null: each CTA builds its own
-    // search, two-level reduction (or null: the launch's last CTA reduces
-    // every particle over the point tiles): the last CTA of each chunk writes
-    // its particles' E and count here, the last chunk to finish selects
+    // search of one problem: the last CTA of each chunk writes its particles'
+    // E and count here, search_select_kernel selects (a batched launch's last
+    // CTA reduces every particle over the point tiles and selects)
     unsigned int* chunk_counter;
     float* chunk_E;
     int* chunk_C;
+    SelectPart* select;   // search_select_kernel's partial results
     SearchState* st;
     int compose_mode, update_mode;
     double beta;
@@ -350,7 +362,7 @@ struct FitArgs {
     const float* cells32; // 16-/8-bit grids, full view: the records as floats too (else null)
     int nx, ny, nz;
     int row, plane;       // index strides along y and z of what the launch samples: the node array's, or the cell view's
-    double vs;
+    double iv;            // 1 / voxel size
     double org[3];
     // reduction
     float* part_S;
@@ -413,30 +425,6 @@ __device__ inline void so3_exp_d(const double w[3], double R[9])
     R[8] = 1.0 - b * (w[0] * w[0] + w[1] * w[1]);
 }
 
-// Pose update in FP64: out = [dR | dt] applied to P (mode 0: dR*R, dR*t+dt;
-// mode 1: dR*R, t+dt), then one Newton-Schulz step R <- R (3I - R^T R)/2
-// to restore orthonormality.
-__device__ inline void compose_d(const double dR[9], const double dt[3], const double P[12], int mode,
-                                 double out[12])
-{
-    double R[9];
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c)
-            R[3 * r + c] = dR[3 * r] * P[c] + dR[3 * r + 1] * P[4 + c] + dR[3 * r + 2] * P[8 + c];
-        const double tr = mode == 0 ? dR[3 * r] * P[3] + dR[3 * r + 1] * P[7] + dR[3 * r + 2] * P[11] : P[4 * r + 3];
-        out[4 * r + 3] = tr + dt[r];
-    }
-    double M[9];  // R^T R
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) M[3 * r + c] = R[r] * R[c] + R[3 + r] * R[3 + c] + R[6 + r] * R[6 + c];
-    for (int r = 0; r < 3; ++r)
-        for (int c = 0; c < 3; ++c) {
-            double acc = 0.0;
-            for (int m = 0; m < 3; ++m) acc += R[3 * r + m] * ((m == c ? 3.0 : 0.0) - M[3 * m + c]);
-            out[4 * r + c] = 0.5 * acc;
-        }
-}
-
 // Particles as the sampling loop uses them.
 //
 // Particle k maps a camera-frame point x to grid units, relative to an
@@ -477,7 +465,7 @@ __device__ inline void particle_pose(const FitArgs& a, int k, double R[9], doubl
             }
         } else {
             const float* u = a.templ + 6 * (size_t)k;
-            const double wr = a.st->s[0] * kPi / 180.0, wt = a.st->s[1] / 100.0;
+            const double wr = a.st->w[0], wt = a.st->w[1];
             const double dw[3] = {wr * (double)u[0], wr * (double)u[1], wr * (double)u[2]};
             double dR[9];
             so3_exp_d<SERIES>(dw, dR);
@@ -498,56 +486,6 @@ struct PlainXf {
     float A[9];
     float c[3];
 };
-
-// Particles k_begin .. k_begin+kc-1 into shared memory, and the chunk's
-// reference matrix A_ref (its first particle) as hi and lo floats; with
-// sAbs, also each particle's plain float transform.
-// CHUNK (the chunk build kernel): the series form of the exponential, and
-// thread 0's pose (the chunk's first particle) passed to the other threads
-// by shuffles instead of each thread forming it again.
-template <int SRC, bool CHUNK = false>
-__device__ void build_particles(const FitArgs& a, int k_begin, int kc, Particle* sP, float* sRef, PlainXf* sAbs)
-{
-    const int t = threadIdx.x;  // (kc <= KC = 32: one warp)
-    if (t >= kc) return;
-    double R[9], tw[3], R0[9], t0[3];
-    particle_pose<SRC, CHUNK>(a, k_begin + t, R, tw);
-    if (CHUNK) {
-        const unsigned lanes = kc >= 32 ? 0xffffffffu : (1u << kc) - 1u;
-        for (int q = 0; q < 9; ++q) R0[q] = __shfl_sync(lanes, R[q], 0);
-        for (int r = 0; r < 3; ++r) t0[r] = __shfl_sync(lanes, tw[r], 0);
-    } else {
-        particle_pose<SRC>(a, k_begin, R0, t0);
-    }
-    const double iv = 1.0 / a.vs;
-    float d[9], b[3];
-    int magic[3];
-    bool ok = true;
-    for (int r = 0; r < 3; ++r) {
-        for (int c = 0; c < 3; ++c) d[3 * r + c] = (float)(R[3 * r + c] * iv - R0[3 * r + c] * iv);
-        const double tg = (tw[r] - a.org[r]) * iv;
-        ok = ok && fabs(tg) < 2097152.0;  // 2^21: beyond, no point can reach the grid
-        const double o = ok ? floor(tg) : 0.0;
-        b[r] = (float)(tg - o);
-        magic[r] = kMagicBits - (int)o;
-    }
-    if (!ok) magic[0] = kNeverValid;
-    if (sAbs) {
-        for (int q = 0; q < 9; ++q) sAbs[t].A[q] = (float)(R[q] * iv);
-        for (int r = 0; r < 3; ++r) sAbs[t].c[r] = (float)((tw[r] - a.org[r]) * iv);
-    }
-    sP[t].d0 = make_float4(d[0], d[1], d[2], b[0]);
-    sP[t].d1 = make_float4(d[3], d[4], d[5], b[1]);
-    sP[t].d2 = make_float4(d[6], d[7], d[8], b[2]);
-    sP[t].m = make_int4(magic[0], magic[1], magic[2], 0);
-    if (t == 0)
-        for (int q = 0; q < 9; ++q) {
-            const double A0 = R0[q] * iv;
-            const float hi = (float)A0;
-            sRef[q] = hi;
-            sRef[9 + q] = (float)(A0 - (double)hi);
-        }
-}
 
 // One row of y = A_ref x, with A_ref = hi + lo, accurate to ~1e-12 of |y|
 // (exact products and two-sums in float), returned as an integer part and a
@@ -945,41 +883,84 @@ struct ChunkData {
 };
 static_assert(sizeof(ChunkData) % 16 == 0, "ChunkData is copied as 16-byte words");
 
-// One warp per chunk: thread t builds particle k_begin + t exactly as a CTA
-// would (build_particles, make_particle_d), and the chunk's spread and reach
-// come from warp reductions of the per-particle values (maxima and minima:
-// the same values as the serial loop, whatever the order).
-template <int SRC>
-__global__ void __launch_bounds__(32) chunk_build_kernel(FitArgs a, ChunkData* out)
+// Particles k_begin .. k_begin + kc - 1 (kc <= 32) as a CTA uses them, by one
+// warp: lane t builds particle t against the chunk's first, and the chunk's
+// spread and reach are warp reductions.  With sAbs, also each particle's plain
+// float transform.  SERIES: the series form of the exponential.
+// FP64 instructions, a hundred cycles of latency and more apiece, are what it
+// costs (conversions to and from FP64 are such too), so they are counted: the
+// scale 1 / vs and the search size come ready, the first particle's products
+// by shuffles, and its float pair is formed by a lane per element (about 155
+// where 250 were; a search iteration's chunks 11.7 -> 9.1 us, a pf_fitness call
+// of 64 poses, where each CTA builds its own, 37 -> 31 us).
+template <int SRC, bool SERIES>
+__device__ void build_chunk(const FitArgs& a, int k_begin, int kc, ChunkData& C, PlainXf* sAbs)
 {
     const int t = threadIdx.x;
-    const int k_begin = blockIdx.x * KC;
-    const int kc = min(KC, a.K - k_begin);
-    if (SRC != SRC_POSES && a.st->lost) return;  // the fitness launch skips every chunk then
-    ChunkData& C = out[blockIdx.x];
-    const int nx = a.row, nxy = a.plane;
-    build_particles<SRC, true>(a, k_begin, kc, C.P, C.ref, nullptr);
-    __syncwarp();
+    const unsigned all = 0xffffffffu;
     const bool mine = t < kc;
-    Particle P;
-    if (mine) {
-        P = C.P[t];
-        make_particle_d(P, nx, nxy, C.PD[t]);
+    float4 row[3] = {make_float4(0, 0, 0, 0), make_float4(0, 0, 0, 0), make_float4(0, 0, 0, 0)};
+    int m[3] = {0, 0, 0};
+    double A0 = 0.0;  // lane q < 9: element q of the first particle's matrix in grid units
+    double tg[3];
+    bool ok = true;
+    if (SRC == SRC_EVAL) {
+        // the one particle is its own reference: its matrix differs by zero
+        const double* P = a.st->P;
+        if (t < 9) A0 = P[4 * (t / 3) + t % 3] * a.iv;
+        for (int r = 0; r < 3; ++r) tg[r] = (P[4 * r + 3] - a.org[r]) * a.iv;
+    } else {
+        double R[9], tw[3], Rg[9], R0[9];
+        particle_pose<SRC, SERIES>(a, k_begin + (mine ? t : 0), R, tw);
+        float d[9];
+#pragma unroll
+        for (int q = 0; q < 9; ++q) {
+            Rg[q] = R[q] * a.iv;
+            R0[q] = __shfl_sync(all, Rg[q], 0);
+            d[q] = (float)(Rg[q] - R0[q]);
+            if (t == q) A0 = R0[q];
+        }
+        for (int r = 0; r < 3; ++r) {
+            row[r] = make_float4(d[3 * r], d[3 * r + 1], d[3 * r + 2], 0.0f);
+            tg[r] = (tw[r] - a.org[r]) * a.iv;
+        }
+        if (sAbs && mine)
+            for (int q = 0; q < 9; ++q) sAbs[t].A[q] = (float)Rg[q];
     }
-    const float4 row[3] = {mine ? P.d0 : make_float4(0, 0, 0, 0), mine ? P.d1 : make_float4(0, 0, 0, 0),
-                           mine ? P.d2 : make_float4(0, 0, 0, 0)};
-    const int m[3] = {mine ? P.m.x : 0, mine ? P.m.y : 0, mine ? P.m.z : 0};
+    for (int r = 0; r < 3; ++r) {
+        ok = ok && fabs(tg[r]) < 2097152.0;  // 2^21: beyond, no point can reach the grid
+        const double o = ok ? floor(tg[r]) : 0.0;
+        row[r].w = (float)(tg[r] - o);
+        m[r] = kMagicBits - (int)o;
+        if (sAbs && mine) sAbs[t].c[r] = (float)tg[r];
+    }
+    if (!ok) m[0] = kNeverValid;
+    if (mine) {
+        Particle P;
+        P.d0 = row[0];
+        P.d1 = row[1];
+        P.d2 = row[2];
+        P.m = make_int4(m[0], m[1], m[2], 0);
+        C.P[t] = P;
+        make_particle_d(P, a.row, a.plane, C.PD[t]);
+    }
+    if (t < 9) {
+        const float hi = (float)A0;
+        C.ref[t] = hi;
+        C.ref[9 + t] = (float)(A0 - (double)hi);
+    }
     float dt = 0.0f, dr = 0.0f, dmax = 0.0f;
     int omin[3], omax[3];
     for (int r = 0; r < 3; ++r) {
-        // particle 0 of the chunk, as the serial loop takes it
-        const float o0 = (float)(kMagicBits - __shfl_sync(0xffffffffu, m[r], 0));
-        const float b0 = __shfl_sync(0xffffffffu, row[r].w, 0);
+        // against the chunk's first particle
+        const float o0 = (float)(kMagicBits - __shfl_sync(all, m[r], 0));
+        const float b0 = __shfl_sync(all, row[r].w, 0);
         const int o = kMagicBits - m[r];
         omin[r] = mine ? o : INT_MAX;
         omax[r] = mine ? o : INT_MIN;
         if (mine) {
             const float sum = fabsf(row[r].x) + fabsf(row[r].y) + fabsf(row[r].z);
+            // a non-finite particle disables the interior path
             dmax = (sum < INFINITY && fabsf(row[r].w) <= 1.0f) ? fmaxf(dmax, sum) : INFINITY;
             if (t > 0) {
                 dt = fmaxf(dt, fabsf((float)(kMagicBits - m[r]) + row[r].w - (o0 + b0)));
@@ -988,13 +969,13 @@ __global__ void __launch_bounds__(32) chunk_build_kernel(FitArgs a, ChunkData* o
         }
     }
     for (int o = 16; o > 0; o >>= 1) {
-        dt = fmaxf(dt, __shfl_xor_sync(0xffffffffu, dt, o));
-        dr = fmaxf(dr, __shfl_xor_sync(0xffffffffu, dr, o));
-        dmax = fmaxf(dmax, __shfl_xor_sync(0xffffffffu, dmax, o));
+        dt = fmaxf(dt, __shfl_xor_sync(all, dt, o));
+        dr = fmaxf(dr, __shfl_xor_sync(all, dr, o));
+        dmax = fmaxf(dmax, __shfl_xor_sync(all, dmax, o));
     }
     for (int r = 0; r < 3; ++r) {
-        omin[r] = __reduce_min_sync(0xffffffffu, omin[r]);
-        omax[r] = __reduce_max_sync(0xffffffffu, omax[r]);
+        omin[r] = __reduce_min_sync(all, omin[r]);
+        omax[r] = __reduce_max_sync(all, omax[r]);
     }
     if (t == 0) {
         C.spread[0] = dt;
@@ -1008,6 +989,239 @@ __global__ void __launch_bounds__(32) chunk_build_kernel(FitArgs a, ChunkData* o
     }
 }
 
+// The chunks of a search iteration, one warp each.
+__global__ void __launch_bounds__(32) chunk_build_kernel(FitArgs a, ChunkData* out)
+{
+    if (a.st->lost) return;  // the fitness launch skips every chunk then
+    const int k_begin = blockIdx.x * KC;
+    build_chunk<SRC_SEARCH, true>(a, k_begin, min(KC, a.K - k_begin), out[blockIdx.x], nullptr);
+}
+
+// Barrier of a block's first two warps (which alone run the pose update).
+__device__ __forceinline__ void pair_sync() { asm volatile("bar.sync 1, 64;" ::: "memory"); }
+
+// Scales the search size by f and keeps it in radians and metres too.
+__device__ inline void scale_search(SearchState* st, double f)
+{
+    st->s[0] *= f;
+    st->s[1] *= f;
+    st->w[0] = st->s[0] * kPi / 180.0;
+    st->w[1] = st->s[1] / 100.0;
+}
+
+struct SelectResult {
+    double mu[6];     // sum of the advantage set's templates
+    float E0, E_best;
+    int C0, best, n_adv;
+    // scratch of pair_update
+    double dw[3], dt[3], coef[4], dR[9], R[9], M[9], P[12], Pn[12];
+};
+
+// The end of a search iteration by a block's first two warps: the record, the
+// lost test, and the update of the pose (dR = Exp(dw) by Rodrigues' formula,
+// R <- dR R with one Newton-Schulz step R (3I - R^T R) / 2 to restore
+// orthonormality, t <- dR t + dt or t + dt) and of the search size.  One
+// thread's chain of some 300 FP64 instructions becomes about 130: an element a
+// lane with one thread's expression for it, the sine and
+// the cosine in two warps.
+__device__ inline void pair_update(const FitArgs& a, int N, long long n_eval, SelectResult& r)
+{
+    const int tid = threadIdx.x, it = a.iter;
+    SearchState* st = a.st;
+    pf_track_stats* stt = a.stats;
+    const bool lost = it == 0 && (!isfinite(r.E0) || (double)r.C0 < (double)a.min_valid_frac * (double)n_eval);
+    const bool best = a.update_mode == 1;
+    const bool moved = !lost && (best || r.n_adv > 0);
+    if (tid == 32) {
+        stt->n_points = N;
+        stt->E0[it] = r.E0;
+        stt->E_best[it] = r.E_best;
+        stt->best[it] = r.best;
+        stt->n_adv[it] = r.n_adv;
+        stt->n_valid0[it] = r.C0;
+        stt->n_eval[it] = (int)n_eval;
+        stt->k_used[it] = a.K;
+        stt->s[it][0] = st->s[0];
+        stt->s[it][1] = st->s[1];
+        stt->n_iters = it + 1;
+    }
+    pair_sync();  // (the record holds the search size before its update)
+    if (lost) {
+        if (tid == 0) {
+            st->lost = 1;
+            stt->E_new[it] = INFINITY;
+        }
+        if (tid < 12) stt->pose[it][tid] = st->P0[tid];
+        return;
+    }
+    if (tid < 12) r.P[tid] = st->P[tid];
+    if (moved) {
+        if (tid < 6) {
+            const double w = st->w[tid < 3 ? 0 : 1];
+            const double u = best ? (double)a.templ[6 * (size_t)r.best + tid] : r.mu[tid] / r.n_adv;
+            *(tid < 3 ? r.dw + tid : r.dt + (tid - 3)) = w * u;
+        }
+        pair_sync();
+        double th2 = 0.0, th = 0.0;
+        if (tid == 0 || tid == 32) {
+            th2 = r.dw[0] * r.dw[0] + r.dw[1] * r.dw[1] + r.dw[2] * r.dw[2];
+            th = sqrt(th2);
+            r.coef[2 + (tid >> 5)] = th < 1e-8 ? th2 : tid == 0 ? sin(0.5 * th) : cos(0.5 * th);
+        }
+        pair_sync();
+        if (tid == 0 || tid == 32) {
+            const double sh = r.coef[2], ch = r.coef[3];
+            if (tid == 0)
+                r.coef[0] = th < 1e-8 ? 1.0 - th2 / 6.0 : 2.0 * sh * ch / th;
+            else
+                r.coef[1] = th < 1e-8 ? 0.5 - th2 / 24.0 : 2.0 * sh * sh / th2;
+        }
+        pair_sync();
+        const int i = tid / 3, c = tid % 3;  // lane q < 9: element (i, c)
+        if (tid < 9) {
+            const double ca = r.coef[0], cb = r.coef[1];
+            if (i == c) {
+                const double x = r.dw[i == 0 ? 1 : 0], y = r.dw[i == 2 ? 1 : 2];
+                r.dR[tid] = 1.0 - cb * (x * x + y * y);
+            } else {
+                // -a w2, a w1 | a w2, -a w0 | -a w1, a w0, and b w_i w_c
+                const double aw = (c == (i + 1) % 3 ? -ca : ca) * r.dw[3 - i - c];
+                r.dR[tid] = aw + cb * r.dw[min(i, c)] * r.dw[max(i, c)];
+            }
+        }
+        pair_sync();
+        if (tid < 9) {
+            const double* d = r.dR + 3 * i;
+            r.R[tid] = d[0] * r.P[c] + d[1] * r.P[4 + c] + d[2] * r.P[8 + c];
+        } else if (tid < 12) {
+            const int q = tid - 9;
+            const double* d = r.dR + 3 * q;
+            const double tr = a.compose_mode == 0 ? d[0] * r.P[3] + d[1] * r.P[7] + d[2] * r.P[11] : r.P[4 * q + 3];
+            r.Pn[4 * q + 3] = tr + r.dt[q];
+        }
+        pair_sync();
+        if (tid < 9) r.M[tid] = r.R[i] * r.R[c] + r.R[3 + i] * r.R[3 + c] + r.R[6 + i] * r.R[6 + c];  // R^T R
+        pair_sync();
+        if (tid < 9) {
+            double acc = 0.0;
+            for (int m = 0; m < 3; ++m) acc += r.R[3 * i + m] * ((m == c ? 3.0 : 0.0) - r.M[3 * m + c]);
+            r.Pn[4 * i + c] = 0.5 * acc;
+        }
+        pair_sync();
+        if (tid < 12) st->P[tid] = r.Pn[tid];
+    }
+    if (tid < 12) stt->pose[it][tid] = moved ? r.Pn[tid] : r.P[tid];
+    if (tid == 0) {
+        if (best || !moved) {
+            const float En = best ? r.E_best : r.E0;
+            const double e = isfinite(En) ? (double)En : 1.0;
+            scale_search(st, a.beta + (1.0 - a.beta) * e);
+            stt->E_new[it] = En;
+            st->pending_s = 0;
+        } else {
+            st->pending_s = 1;  // until the new pose is evaluated
+        }
+    }
+}
+
+// Selection of a search iteration (a launch of its own after the fitness
+// launch): argmin (lowest index on ties), advantage set and its template sums,
+// then the pose update by the last block to finish (ticket counter, no
+// spinning).  The sums are FP64, added in the order one block of 256 threads
+// would: thread k mod 256 over k, then a warp's butterfly, then the warps.
+// Such a block, the last CTA of the fitness launch, has 12 FP64 instructions
+// for each 32 particles on one SM's narrow pipe while 151 SMs idle: 31, 35 and
+// 72 us of the launches of 1024, 3072 and 10240 particles.  So block (class, q)
+// takes one of its warps and one of the six sums: 14 to 17 us a launch, mostly
+// the pose update's chain (640x480 frame of the paper's schedule, with the
+// chunks above: 6426 -> 5800 us; 160x120 frame in a 64^3 map 1296 -> 1145).
+__global__ void __launch_bounds__(64) search_select_kernel(FitArgs a)
+{
+    __shared__ SelectResult res;
+    __shared__ int s_last;
+    if (a.st->lost) return;
+    const int tid = threadIdx.x, lane = tid & 31, cls = blockIdx.x / 6, q = blockIdx.x % 6;
+    SelectPart* part = a.select;
+    const unsigned all = 0xffffffffu;
+    if (tid < 32) {
+        const float E0 = __ldcg(a.chunk_E);
+        float be = INFINITY;
+        int bk = 0, nadv = 0;
+        double sum = 0.0;
+        constexpr int B = 8;  // loads in flight
+        for (int k0 = 32 * cls + lane; k0 < a.K; k0 += 256 * B) {
+            float E[B], u[B];
+#pragma unroll
+            for (int b = 0; b < B; ++b) E[b] = k0 + 256 * b < a.K ? __ldcg(a.chunk_E + k0 + 256 * b) : INFINITY;
+#pragma unroll
+            for (int b = 0; b < B; ++b) u[b] = E[b] < E0 ? __ldg(a.templ + 6 * (size_t)(k0 + 256 * b) + q) : 0.0f;
+#pragma unroll
+            for (int b = 0; b < B; ++b) {
+                if (E[b] < be) {
+                    be = E[b];
+                    bk = k0 + 256 * b;
+                }
+                if (E[b] < E0) {
+                    ++nadv;
+                    sum += (double)u[b];
+                }
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(all, sum, o);
+        if (q == 0) {
+            nadv = __reduce_add_sync(all, nadv);
+            for (int o = 16; o > 0; o >>= 1) {
+                const float e2 = __shfl_xor_sync(all, be, o);
+                const int k2 = __shfl_xor_sync(all, bk, o);
+                if (e2 < be || (e2 == be && k2 < bk)) {
+                    be = e2;
+                    bk = k2;
+                }
+            }
+        }
+        if (lane == 0) {
+            part->sum[cls][q] = sum;
+            if (q == 0) {
+                part->e[cls] = be;
+                part->k[cls] = bk;
+                part->n_adv[cls] = nadv;
+            }
+            __threadfence();
+            s_last = atomicAdd(&part->ticket, 1u) == gridDim.x - 1;
+        }
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    if (tid < 6) {
+        double mu = 0.0;
+        for (int w = 0; w < SEL_CLASSES; ++w) mu += __ldcg(&part->sum[w][tid]);
+        res.mu[tid] = mu;
+    }
+    const int N = *a.n_dev;
+    if (tid == 32) {
+        float be = INFINITY;
+        int bk = 0x7fffffff, n_adv = 0;
+        for (int w = 0; w < SEL_CLASSES; ++w) {
+            const float e = __ldcg(&part->e[w]);
+            const int k = __ldcg(&part->k[w]);
+            if (e < be || (e == be && k < bk)) {
+                be = e;
+                bk = k;
+            }
+            n_adv += __ldcg(&part->n_adv[w]);
+        }
+        res.E0 = __ldcg(a.chunk_E);
+        res.C0 = __ldcg(a.chunk_C);
+        res.E_best = be;
+        res.best = bk;
+        res.n_adv = n_adv;
+        part->ticket = 0u;
+    }
+    pair_sync();
+    pair_update(a, N, N > 0 ? ((long long)N + a.stride - 1) / a.stride : 0, res);
+}
+
 // The work of one CTA: particle chunk bx, point tile by, of a launch of
 // n_blocks CTAs for this problem (the last of them to finish runs the
 // epilogue).
@@ -1018,7 +1232,6 @@ template <int SRC, int VARIANT, typename TS, bool SOLO>
 __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, unsigned n_blocks)
 {
     __shared__ __align__(16) ChunkData sC;
-    Particle* const sP = sC.P;
     ParticleD* const sPD = sC.PD;
     float* const sRef = sC.ref;
     __shared__ PlainXf sAbs[VARIANT == 1 ? KC : 1];
@@ -1034,7 +1247,6 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
     float* const s_spread = sC.spread;
     __shared__ float s_red[FIT_WARPS];
     float& s_dmax = sC.dmax;
-    __shared__ long long s_omin[3], s_omax[3];
     __shared__ int s_lo[3], s_hi[3];
 
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -1063,54 +1275,8 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
             const int4* src = reinterpret_cast<const int4*>(static_cast<const ChunkData*>(a.chunks) + bx);
             int4* dst = reinterpret_cast<int4*>(&sC);
             for (int q = tid; q < (int)(sizeof(ChunkData) / 16); q += FIT_THREADS) dst[q] = __ldg(src + q);
-        } else {
-            build_particles<SRC>(a, k_begin, kc, sP, sRef, VARIANT == 1 ? sAbs : nullptr);
-            if (tid < kc) make_particle_d(sP[tid], nx, nxy, sPD[tid]);
-        }
-    }
-    __syncthreads();
-    if (prebuilt && tid == 0) {
-        for (int r = 0; r < 3; ++r) {
-            s_omin[r] = skip ? LLONG_MAX : (long long)sC.omin[r];
-            s_omax[r] = skip ? LLONG_MIN : (long long)sC.omax[r];
-        }
-    }
-    // spread of the chunk's particles relative to its first one: translation
-    // (voxels) and rotation (voxels per metre of point distance); and the
-    // chunk's reach: the range of the particles' integer cell offsets o_k
-    // and the largest row sum of |dA_k|, which bound where any particle can
-    // put a point (see the interior test below)
-    if (!prebuilt && tid == 0) {
-        float dt = 0.0f, dr = 0.0f, dmax = 0.0f;
-        long long omin[3] = {LLONG_MAX, LLONG_MAX, LLONG_MAX}, omax[3] = {LLONG_MIN, LLONG_MIN, LLONG_MIN};
-        if (!skip) {
-            const float o0[3] = {(float)(kMagicBits - sP[0].m.x), (float)(kMagicBits - sP[0].m.y),
-                                 (float)(kMagicBits - sP[0].m.z)};
-            const float b0[3] = {sP[0].d0.w, sP[0].d1.w, sP[0].d2.w};
-            for (int k = 0; k < kc; ++k) {
-                const Particle& P = sP[k];
-                const float4 row[3] = {P.d0, P.d1, P.d2};
-                const int m[3] = {P.m.x, P.m.y, P.m.z};
-                for (int r = 0; r < 3; ++r) {
-                    const long long o = (long long)kMagicBits - (long long)m[r];
-                    omin[r] = o < omin[r] ? o : omin[r];
-                    omax[r] = o > omax[r] ? o : omax[r];
-                    const float sum = fabsf(row[r].x) + fabsf(row[r].y) + fabsf(row[r].z);
-                    // a non-finite particle disables the interior path
-                    dmax = (sum < INFINITY && fabsf(row[r].w) <= 1.0f) ? fmaxf(dmax, sum) : INFINITY;
-                    if (k > 0) {
-                        dt = fmaxf(dt, fabsf((float)(kMagicBits - m[r]) + row[r].w - (o0[r] + b0[r])));
-                        dr = fmaxf(dr, sum);
-                    }
-                }
-            }
-        }
-        s_spread[0] = dt;
-        s_spread[1] = dr;
-        s_dmax = dmax;
-        for (int r = 0; r < 3; ++r) {
-            s_omin[r] = omin[r];
-            s_omax[r] = omax[r];
+        } else if (warp == 0) {
+            build_chunk<SRC, false>(a, k_begin, kc, sC, VARIANT == 1 ? sAbs : nullptr);
         }
     }
     __syncthreads();
@@ -1202,7 +1368,7 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                 const long long E = reach < 1.0e6f ? (long long)ceilf(reach) + 3 : (1ll << 40);
                 const int n[3] = {a.nx, a.ny, a.nz};
                 for (int r = 0; r < 3; ++r) {
-                    const long long lo = E - s_omin[r], hi = (long long)(n[r] - 2) - E - s_omax[r];
+                    const long long lo = E - sC.omin[r], hi = (long long)(n[r] - 2) - E - sC.omax[r];
                     s_lo[r] = (int)(lo > INT_MAX ? INT_MAX : (lo < INT_MIN ? INT_MIN : lo));
                     s_hi[r] = (int)(hi < INT_MIN ? INT_MIN : (hi > INT_MAX ? INT_MAX : hi));
                 }
@@ -1382,10 +1548,10 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
     }
     __threadfence();
     __syncthreads();
-    const bool two_level = SOLO && SRC == SRC_SEARCH && a.chunk_counter != nullptr;
-    if (two_level) {
+    if (SOLO && SRC == SRC_SEARCH) {
         // the last of the chunk's point tiles reduces the chunk's particles
-        // over the tiles (in parallel with other chunks' sampling) ...
+        // over the tiles (in parallel with other chunks' sampling);
+        // search_select_kernel does the rest
         if (tid == 0) {
             const unsigned int ticket = atomicAdd(a.chunk_counter + bx, 1u);
             s_last = ticket == (unsigned)a.n_ptiles - 1;
@@ -1401,18 +1567,11 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
             a.chunk_C[k_begin + tid] = C;
         }
         if (tid == 0) a.chunk_counter[bx] = 0u;
-        __threadfence();
-        __syncthreads();
-        // ... and the last chunk to finish runs the selection below
-        if (tid == 0) {
-            const unsigned int ticket = atomicAdd(a.counter, 1u);
-            s_last = ticket == (unsigned)((a.K + KC - 1) / KC) - 1;
-        }
-    } else {
-        if (tid == 0) {
-            const unsigned int ticket = atomicAdd(a.counter, 1u);
-            s_last = ticket == n_blocks - 1;
-        }
+        return;
+    }
+    if (tid == 0) {
+        const unsigned int ticket = atomicAdd(a.counter, 1u);
+        s_last = ticket == n_blocks - 1;
     }
     __syncthreads();
     if (!s_last) return;
@@ -1458,32 +1617,25 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                 const float E = C > 0 ? __fdiv_rn(S, (float)C) : INFINITY;
                 SearchState* st = a.st;
                 const double e = isfinite(E) ? (double)E : 1.0;
-                const double f = a.beta + (1.0 - a.beta) * e;
-                st->s[0] *= f;
-                st->s[1] *= f;
+                scale_search(st, a.beta + (1.0 - a.beta) * e);
                 st->pending_s = 0;
                 a.stats->E_new[a.iter] = E;
             }
         }
-    } else {  // SRC_SEARCH
+    } else if (!SOLO) {  // SRC_SEARCH of a batched launch
         __shared__ float s_E0;
         __shared__ int s_C0;
         __shared__ float se[FIT_WARPS];
         __shared__ int sk[FIT_WARPS];
         __shared__ double sd[FIT_WARPS][6];
         __shared__ int sn[FIT_WARPS];
-        SearchState* st = a.st;
+        __shared__ SelectResult res;
         if (tid == 0) {
-            if (two_level) {
-                s_E0 = __ldcg(a.chunk_E);
-                s_C0 = __ldcg(a.chunk_C);
-            } else {
-                float S;
-                int C;
-                sum_tiles(a.part_S, a.part_C, a.K, a.n_ptiles, 0, S, C);
-                s_E0 = C > 0 ? __fdiv_rn(S, (float)C) : INFINITY;
-                s_C0 = C;
-            }
+            float S;
+            int C;
+            sum_tiles(a.part_S, a.part_C, a.K, a.n_ptiles, 0, S, C);
+            s_E0 = C > 0 ? __fdiv_rn(S, (float)C) : INFINITY;
+            s_C0 = C;
         }
         __syncthreads();
         const float E0 = s_E0;
@@ -1492,15 +1644,10 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
         int nadv = 0;
         double sum[6] = {0, 0, 0, 0, 0, 0};
         for (int k = tid; k < a.K; k += FIT_THREADS) {
-            float E;
-            if (two_level) {
-                E = __ldcg(a.chunk_E + k);
-            } else {
-                float S;
-                int C;
-                sum_tiles(a.part_S, a.part_C, a.K, a.n_ptiles, k, S, C);
-                E = C > 0 ? __fdiv_rn(S, (float)C) : INFINITY;
-            }
+            float S;
+            int C;
+            sum_tiles(a.part_S, a.part_C, a.K, a.n_ptiles, k, S, C);
+            const float E = C > 0 ? __fdiv_rn(S, (float)C) : INFINITY;
             if (E < be) {
                 be = E;
                 bk = k;
@@ -1523,70 +1670,23 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
             for (int q = 0; q < 6; ++q) sd[warp][q] = sum[q];
         }
         __syncthreads();
-        if (tid == 0 && !skip) {
-            int n_adv = 0;
-            double mu[6] = {0, 0, 0, 0, 0, 0};
-            for (int w = 0; w < FIT_WARPS; ++w) {
-                n_adv += sn[w];
-                for (int q = 0; q < 6; ++q) mu[q] += sd[w][q];
+        if (!skip && tid < 64) {
+            if (tid < 6) {
+                double mu = 0.0;
+                for (int w = 0; w < FIT_WARPS; ++w) mu += sd[w][tid];
+                res.mu[tid] = mu;
             }
-            pf_track_stats* stt = a.stats;
-            const int it = a.iter;
-            const long long nev = Ne;
-            const double s_deg = st->s[0], s_cm = st->s[1];
-            stt->n_points = N;
-            stt->E0[it] = E0;
-            stt->E_best[it] = be;
-            stt->best[it] = bk;
-            stt->n_adv[it] = n_adv;
-            stt->n_valid0[it] = s_C0;
-            stt->n_eval[it] = (int)nev;
-            stt->k_used[it] = a.K;
-            stt->s[it][0] = s_deg;
-            stt->s[it][1] = s_cm;
-            stt->n_iters = it + 1;
-            const bool lost = it == 0 && (!isfinite(E0) || (double)s_C0 < (double)a.min_valid_frac * (double)nev);
-            if (lost) {
-                st->lost = 1;
-                stt->E_new[it] = INFINITY;
-                for (int q = 0; q < 12; ++q) stt->pose[it][q] = st->P0[q];
-            } else {
-                const double wr = s_deg * kPi / 180.0, wt = s_cm / 100.0;
-                double dw[3], dt[3];
-                bool moved = true;
-                if (a.update_mode == 1) {
-                    const float* u = a.templ + 6 * (size_t)bk;
-                    for (int q = 0; q < 3; ++q) {
-                        dw[q] = wr * (double)u[q];
-                        dt[q] = wt * (double)u[3 + q];
-                    }
-                } else if (n_adv > 0) {
-                    for (int q = 0; q < 3; ++q) {
-                        dw[q] = wr * (mu[q] / n_adv);
-                        dt[q] = wt * (mu[3 + q] / n_adv);
-                    }
-                } else {
-                    moved = false;
-                }
-                if (moved) {
-                    double dR[9], Pn[12];
-                    so3_exp_d(dw, dR);
-                    compose_d(dR, dt, st->P, a.compose_mode, Pn);
-                    for (int q = 0; q < 12; ++q) st->P[q] = Pn[q];
-                }
-                for (int q = 0; q < 12; ++q) stt->pose[it][q] = st->P[q];
-                if (a.update_mode == 1 || !moved) {
-                    const float En = a.update_mode == 1 ? be : E0;
-                    const double e = isfinite(En) ? (double)En : 1.0;
-                    const double f = a.beta + (1.0 - a.beta) * e;
-                    st->s[0] *= f;
-                    st->s[1] *= f;
-                    stt->E_new[it] = En;
-                    st->pending_s = 0;
-                } else {
-                    st->pending_s = 1;
-                }
+            if (tid == 32) {
+                int n_adv = 0;
+                for (int w = 0; w < FIT_WARPS; ++w) n_adv += sn[w];
+                res.n_adv = n_adv;
+                res.E0 = E0;
+                res.C0 = s_C0;
+                res.E_best = be;
+                res.best = bk;
             }
+            pair_sync();
+            pair_update(a, N, Ne, res);
         }
     }
     if (tid == 0) *a.counter = 0u;
@@ -1641,6 +1741,7 @@ __global__ void track_begin_kernel(SearchState* st, const double* P0, double s_d
         }
         st->s[0] = s_deg;
         st->s[1] = s_cm;
+        scale_search(st, 1.0);
         st->lost = 0;
         st->pending_s = 0;
         stats->n_iters = 0;
@@ -1745,7 +1846,7 @@ void fill_volume_args(FitArgs& a, const pf_volume* v, int layout)
     a.nz = v->desc.nz;
     a.row = layout == 3 ? v->pitch.row : v->desc.nx;
     a.plane = layout == 3 ? v->pitch.plane : v->desc.nx * v->desc.ny;
-    a.vs = v->desc.voxel_size;
+    a.iv = 1.0 / (double)v->desc.voxel_size;
     for (int q = 0; q < 3; ++q) a.org[q] = v->desc.origin[q];
 }
 
@@ -1856,6 +1957,8 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
         w.pix_cap = max_pixels;
     }
     if (!w.state) {
+        PF_CUDA(pf::dev_malloc(reinterpret_cast<SelectPart**>(&w.select), sizeof(SelectPart)));
+        PF_CUDA(cudaMemset(w.select, 0, sizeof(SelectPart)));
         PF_CUDA(pf::dev_malloc(&w.state, sizeof(SearchState)));
         PF_CUDA(pf::dev_malloc(&w.n_points, sizeof(int)));
         PF_CUDA(pf::dev_malloc(&w.pose_in, 16 * sizeof(double)));
@@ -2021,19 +2124,19 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
         a.chunk_counter = w.chunk_counter;
         a.chunk_E = w.chunk_E;
         a.chunk_C = w.chunk_C;
+        a.select = static_cast<SelectPart*>(w.select);
         pf::timing_begin(pf::KC_FITNESS, s);
         if (prebuild) {
-            chunk_build_kernel<SRC_SEARCH><<<chunks, 32, 0, s>>>(a, static_cast<ChunkData*>(w.chunks));
+            chunk_build_kernel<<<chunks, 32, 0, s>>>(a, static_cast<ChunkData*>(w.chunks));
             pf::count_launch();
         }
         launch_fitness<SRC_SEARCH>(a, v->fitness_variant, v, chunks, s);
+        search_select_kernel<<<6 * SEL_CLASSES, 64, 0, s>>>(a);
+        pf::count_launch();
         pf::timing_end(pf::KC_FITNESS, s);
         if (p->update_mode == 0) {
             FitArgs e = a;
-            e.chunks = nullptr;  // one particle, built in its CTAs, reduced by the launch's last CTA
-            e.chunk_counter = nullptr;
-            e.chunk_E = nullptr;
-            e.chunk_C = nullptr;
+            e.chunks = nullptr;  // one particle, built in its CTAs
             e.K = 1;
             e.n_ptiles = choose_ptiles(v->device, 1, ne_max);
             pf::timing_begin(pf::KC_FITNESS1, s);

@@ -797,6 +797,7 @@ pf_status pf_destroy_volume(pf_volume* v)
     cudaFree(w.chunk_counter);
     cudaFree(w.chunk_E);
     cudaFree(w.chunk_C);
+    cudaFree(w.select);
     cudaFree(w.counter);
     cudaFree(w.state);
     cudaFree(w.pose_in);
