@@ -802,6 +802,23 @@ __device__ __forceinline__ int linear_cell(const int* Yi, int nx, int nxy)
     return (int)((unsigned)Yi[0] + (unsigned)nx * (unsigned)Yi[1] + (unsigned)nxy * (unsigned)Yi[2]);
 }
 
+// Warp sums of four values at once, each by the butterfly x += shfl_xor(x, o)
+// over o = 16, 8, 4, 2, 1: at the first two levels (fold) a lane keeps the half
+// of the values that its bit selects and hands over the others, so six shuffles
+// do what twenty would, with the same additions (each pair's two lanes would
+// add the same two numbers) and so the same bits.  With fold<16> of values 0
+// and 1 and of 2 and 3, then fold<8> of the two, the lane ends up with value
+// folded_index(lane).  Shuffles go through the L1 data pipe that bounds lanes on
+// points: 3072 spread poses over 307 200 points 5% faster (3.42 -> 3.25 ms).
+template <int O>
+__device__ __forceinline__ float fold(float v0, float v1, int lane)
+{
+    const bool upper = (lane & O) != 0;
+    return (upper ? v1 : v0) + __shfl_xor_sync(0xffffffffu, upper ? v0 : v1, O);
+}
+
+__device__ __forceinline__ int folded_index(int lane) { return ((lane >> 4) & 1) | ((lane >> 2) & 2); }
+
 // Block-wide argmin of (E, k) with the lowest k among equal E.
 __device__ inline void argmin_pair(float& e, int& k, float* se, int* sk)
 {
@@ -1398,42 +1415,52 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                 P2[h].ylb = linear_cell(Yb, nx, nxy);
             }
             if (!s_mode) {
-                if (__all_sync(0xffffffffu, in_all)) {
-                    for (int kk = 0; kk < kc; ++kk) {
-                        XformD X;
-                        load_xformd(sPD[kk], X);
-                        float s = 0.0f;
-                        int c = 0;
+                // four particles at a time, so that one transposed butterfly
+                // serves their four sums (fold)
+                auto particle = [&](auto checked, int kk, float& s, int& c) {
+                    XformD X;
+                    load_xformd(sPD[kk], X);
+                    s = 0.0f;
+                    c = 0;
 #pragma unroll
-                        for (int h = 0; h < PPT / 2; ++h) {
-                            Cell ca, cb;
-                            locate2<false>(X, nx, nxy, mx, my, mz, P2[h], nullptr, nullptr, ca, cb);
-                            gather<VARIANT, TS, true>(a, nx, nxy, ca, s, c);
-                            gather<VARIANT, TS, true>(a, nx, nxy, cb, s, c);
-                        }
-                        c = __reduce_add_sync(0xffffffffu, c);
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-                        if (lane == 0) {
-                            accS[warp][kk] += s;
-                            accC[warp][kk] += c;
-                        }
-                    }
-                } else {
-                    // some point of the warp may leave the grid: per-sample
-                    // range tests
-                    for (int kk = 0; kk < kc; ++kk) {
-                        XformD X;
-                        load_xformd(sPD[kk], X);
-                        float s = 0.0f;
-                        int c = 0;
-#pragma unroll
-                        for (int h = 0; h < PPT / 2; ++h) {
-                            Cell ca, cb;
+                    for (int h = 0; h < PPT / 2; ++h) {
+                        Cell ca, cb;
+                        if constexpr (decltype(checked)::value)
                             locate2<true>(X, nx, nxy, mx, my, mz, P2[h], Yi[h], Yi[h + 2], ca, cb);
-                            gather<VARIANT, TS, true>(a, nx, nxy, ca, s, c);
-                            gather<VARIANT, TS, true>(a, nx, nxy, cb, s, c);
+                        else
+                            locate2<false>(X, nx, nxy, mx, my, mz, P2[h], nullptr, nullptr, ca, cb);
+                        gather<VARIANT, TS, true>(a, nx, nxy, ca, s, c);
+                        gather<VARIANT, TS, true>(a, nx, nxy, cb, s, c);
+                    }
+                };
+                auto particles = [&](auto checked) {
+                    int kk = 0;
+                    for (; kk + 4 <= kc; kk += 4) {
+                        float s, half = 0.0f, prev = 0.0f;
+                        unsigned c4 = 0u;
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            int c;
+                            particle(checked, kk + v, s, c);
+                            c4 |= (unsigned)c << (8 * v);  // (at most 128 a warp)
+                            if (v & 1) s = fold<16>(prev, s, lane);
+                            if (v == 1) half = s;
+                            prev = s;
                         }
+                        s = fold<8>(half, s, lane);
+#pragma unroll
+                        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+                        c4 = __reduce_add_sync(0xffffffffu, c4);
+                        if ((lane & 7) == 0) {
+                            const int v = folded_index(lane);
+                            accS[warp][kk + v] += s;
+                            accC[warp][kk + v] += (c4 >> (8 * v)) & 0xff;
+                        }
+                    }
+                    for (; kk < kc; ++kk) {
+                        float s;
+                        int c;
+                        particle(checked, kk, s, c);
                         c = __reduce_add_sync(0xffffffffu, c);
 #pragma unroll
                         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -1442,7 +1469,12 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                             accC[warp][kk] += c;
                         }
                     }
-                }
+                };
+                // (some point of the warp may leave the grid: per-sample range tests)
+                if (__all_sync(0xffffffffu, in_all))
+                    particles(std::false_type{});
+                else
+                    particles(std::true_type{});
             } else {
                 // the warp's 128 points as 64 pairs: pair h * 32 + lane holds
                 // this lane's points h and h + 2
