@@ -793,7 +793,7 @@ __device__ __forceinline__ bool point_interior(const int* Yi, const float* Yf, c
 {
     bool in = true;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) in = in && Yi[q] >= lo[q] && Yi[q] <= hi[q] && fabsf(Yf[q]) <= 1.0f;
+    for (int q = 0; q < 3; ++q) in = in && Yi[q] >= lo[q] && Yi[q] <= hi[q] && fabsf(Yf[q]) <= 0.505f;
     return in;
 }
 
@@ -1245,7 +1245,8 @@ __global__ void __launch_bounds__(64) search_select_kernel(FitArgs a)
 // SOLO: a launch of one problem, which may use prebuilt particle chunks and
 // the two-level reduction (FitArgs.chunks, .chunk_counter); the batched
 // launch compiles without them.
-template <int SRC, int VARIANT, typename TS, bool SOLO>
+// CTAS: see fitness_kernel.
+template <int SRC, int VARIANT, typename TS, bool SOLO, int CTAS = PF_FIT_MIN_BLOCKS>
 __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, unsigned n_blocks)
 {
     __shared__ __align__(16) ChunkData sC;
@@ -1286,9 +1287,9 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
     }
     __syncthreads();
     const bool skip = s_skip != 0;
-    const bool prebuilt = SOLO && SRC == SRC_SEARCH && a.chunks != nullptr;  // (never with the plain layout)
+    constexpr bool prebuilt = SOLO && SRC == SRC_SEARCH && VARIANT != 1;  // chunk_build_kernel has built the chunks
     if (!skip) {
-        if (prebuilt) {
+        if constexpr (prebuilt) {
             const int4* src = reinterpret_cast<const int4*>(static_cast<const ChunkData*>(a.chunks) + bx);
             int4* dst = reinterpret_cast<int4*>(&sC);
             for (int q = tid; q < (int)(sizeof(ChunkData) / 16); q += FIT_THREADS) dst[q] = __ldg(src + q);
@@ -1376,13 +1377,17 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                 s_mode = kc >= 24 && (s_spread[0] + s_spread[1] * rad) < a.pm_threshold;
                 // Interior test.  Sample cell coordinate on axis r:
                 // yi_r + o_k,r + floor(dA_k,r . x + yf_r + b_k,r) with
-                // |yf| <= 1/2 + eps, 0 <= b < 1 and |dA_k,r . x| <= dmax |x|,
-                // so it lies within yi_r + [omin_r - E, omax_r + E] for
-                // E = ceil(dmax |x|) + 3 (one cell of margin).  A point whose
-                // yi_r keeps that range inside [0, n_r - 2] on every axis
-                // needs no range test under any particle of the chunk.
+                // |yf| <= 0.505 (point_interior asks for it), 0 <= b <= 1 and
+                // |dA_k,r . x| <= dmax |x| = reach, so it lies within
+                // yi_r + [omin_r - E, omax_r + E] for E = floor(reach + 1.52)
+                // (0.015 of a cell for rounding).  A point whose yi_r keeps
+                // that range inside [0, n_r - 2] on every axis needs no range
+                // test under any particle of the chunk.  (Two cells more on
+                // each side left most points of a 64^3 room, whose walls lie
+                // four cells inside the grid, to the tested paths: a 160x120
+                // frame's search there 1100 -> 1008 us.)
                 const float reach = s_dmax * rad;
-                const long long E = reach < 1.0e6f ? (long long)ceilf(reach) + 3 : (1ll << 40);
+                const long long E = reach < 1.0e6f ? (long long)floorf(fmaf(reach, 1.0001f, 1.52f)) : (1ll << 40);
                 const int n[3] = {a.nx, a.ny, a.nz};
                 for (int r = 0; r < 3; ++r) {
                     const long long lo = E - sC.omin[r], hi = (long long)(n[r] - 2) - E - sC.omax[r];
@@ -1518,6 +1523,41 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                             locate2<false>(X, nx, nxy, mx, my, mz, pp, nullptr, nullptr, ca, cb);
                             gather<VARIANT, TS, true, FC>(a, nx, nxy, ca, s, c);
                             gather<VARIANT, TS, true, FC>(a, nx, nxy, cb, s, c);
+                        }
+                    } else if constexpr (CTAS == 1) {
+#pragma unroll 1
+                        for (int j = 0; j < PPT * 16; j += 2) {
+                            // two pairs' cells, then their four records together
+                            Cell cell[4];
+#pragma unroll
+                            for (int u = 0; u < 2; ++u) {
+                                const float4 q0 = sPair[warp][j + u][0], q1 = sPair[warp][j + u][1],
+                                             q2 = sPair[warp][j + u][2];
+                                const int2 yl = sPyl[warp][j + u];
+                                PointPair pp;
+                                pp.x = make_float2(q0.x, q0.y);
+                                pp.y = make_float2(q0.z, q0.w);
+                                pp.z = make_float2(q1.x, q1.y);
+                                pp.yf0 = make_float2(q1.z, q1.w);
+                                pp.yf1 = make_float2(q2.x, q2.y);
+                                pp.yf2 = make_float2(q2.z, q2.w);
+                                pp.yla = yl.x;
+                                pp.ylb = yl.y;
+                                if (yl.x != INT_MIN) {  // the same for every lane
+                                    locate2<false>(X, nx, nxy, mx, my, mz, pp, nullptr, nullptr, cell[2 * u],
+                                                   cell[2 * u + 1]);
+                                } else {
+                                    // a pair near the grid's edge (rare): the
+                                    // reference cells again, from the points
+                                    int Ya[3], Yb[3];
+                                    float Fa[3], Fb[3];
+                                    ref_apply(sRef, pp.x.x, pp.y.x, pp.z.x, Ya, Fa);
+                                    ref_apply(sRef, pp.x.y, pp.y.y, pp.z.y, Yb, Fb);
+                                    locate2<true>(X, nx, nxy, mx, my, mz, pp, Ya, Yb, cell[2 * u], cell[2 * u + 1]);
+                                }
+                            }
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) gather<VARIANT, TS, true, FC>(a, nx, nxy, cell[u], s, c);
                         }
                     } else {
 #pragma unroll 2
@@ -1724,10 +1764,164 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
     if (tid == 0) *a.counter = 0u;
 }
 
-template <int SRC, int VARIANT, typename TS>
-__global__ void __launch_bounds__(FIT_THREADS, PF_FIT_MIN_BLOCKS) fitness_kernel(FitArgs a)
+// CTAS: resident CTAs an SM that the registers are shared among.  A launch with
+// no more CTAs than SMs takes the form for one, whose lanes on particles load
+// the records of two pairs together where some need the range test: 24 warps
+// an SM hide one pair's wait, 8 do not (64 poses over 18 800 points of a 64^3
+// grid, 38 CTAs: 30.8 -> 26.7 us; with 80 registers the two pairs cost a full
+// launch 2%).  The same operations in the same order: the same bits.
+template <int SRC, int VARIANT, typename TS, int CTAS = PF_FIT_MIN_BLOCKS>
+__global__ void __launch_bounds__(FIT_THREADS, CTAS) fitness_kernel(FitArgs a)
 {
-    fitness_body<SRC, VARIANT, TS, true>(a, blockIdx.x, blockIdx.y, gridDim.x * gridDim.y);
+    fitness_body<SRC, VARIANT, TS, true, CTAS>(a, blockIdx.x, blockIdx.y, gridDim.x * gridDim.y);
+}
+
+// Fitness of the updated pose (one particle) over the points of a search of
+// one problem, then the search size: the sums of fitness_body for a chunk of
+// one particle, without its chunk.  The particle is its own reference, so its
+// matrix differs by zero and a sample's offset is y's fraction plus b.  Bound by
+// the latency of its chain; every load that needs no other goes out first, the
+// matrix elements are a thread each (20 evaluations of a 640x480 frame of the
+// paper's schedule 60 us less than by the search's kernel, ten of a 160x120
+// frame 20 us less).
+template <int VARIANT, typename TS>
+__global__ void __launch_bounds__(FIT_THREADS, 2) search_eval_kernel(FitArgs a)
+{
+    __shared__ float s_ref[18], s_b[3], accS[FIT_WARPS];
+    __shared__ int s_magic[3], s_never, accC[FIT_WARPS], s_last;
+    __shared__ PlainXf s_abs;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, by = blockIdx.x;
+    SearchState* st = a.st;
+    const int N = *a.n_dev;
+    const bool skip = st->lost || !st->pending_s;
+    const long long Ne = N > 0 ? ((long long)N + a.stride - 1) / a.stride : 0;
+    const long long beg = Ne * by / a.n_ptiles, end = Ne * (by + 1) / a.n_ptiles;
+    if (tid == 0) s_never = 0;
+    __syncthreads();
+    if (tid < 9) {
+        const double A0 = st->P[4 * (tid / 3) + tid % 3] * a.iv;
+        const float hi = (float)A0;
+        s_ref[tid] = hi;
+        s_ref[9 + tid] = (float)(A0 - (double)hi);
+        s_abs.A[tid] = hi;
+    } else if (tid >= 32 && tid < 35) {
+        const int r = tid - 32;
+        const double tg = (st->P[4 * r + 3] - a.org[r]) * a.iv;
+        const bool ok = fabs(tg) < 2097152.0;  // 2^21: beyond, no point can reach the grid
+        const double o = ok ? floor(tg) : 0.0;
+        s_b[r] = (float)(tg - o);
+        s_magic[r] = kMagicBits - (int)o;
+        s_abs.c[r] = (float)tg;
+        if (!ok) s_never = 1;
+    }
+    if (lane == 0) {
+        accS[warp] = 0.0f;
+        accC[warp] = 0;
+    }
+    __syncthreads();
+    const int row = a.row, plane = a.plane;
+    const int mg[3] = {s_never ? kNeverValid : s_magic[0], s_magic[1], s_magic[2]};
+    for (long long sub = beg; sub < end && !skip; sub += SUBTILE) {
+        float4 q[PPT];
+#pragma unroll
+        for (int p = 0; p < PPT; ++p) {
+            const long long e = sub + p * FIT_THREADS + tid;
+            q[p] = e < end ? __ldg(a.pts + e * a.stride) : make_float4(NAN, NAN, NAN, 0.0f);
+        }
+        float s = 0.0f;
+        int c = 0;
+#pragma unroll
+        for (int i = 0; i < PPT; ++i) {
+            // the pairs' order (0, 2), (1, 3); the plain form's 0, 1, 2, 3
+            const int p = VARIANT == 1 ? i : (i >> 1) + 2 * (i & 1);
+            Cell cell;
+            if (VARIANT == 1) {
+                const PlainXf& X = s_abs;
+                const float gx = fmaf(X.A[0], q[p].x, fmaf(X.A[1], q[p].y, fmaf(X.A[2], q[p].z, X.c[0])));
+                const float gy = fmaf(X.A[3], q[p].x, fmaf(X.A[4], q[p].y, fmaf(X.A[5], q[p].z, X.c[1])));
+                const float gz = fmaf(X.A[6], q[p].x, fmaf(X.A[7], q[p].y, fmaf(X.A[8], q[p].z, X.c[2])));
+                cell.ok = gx >= 0.0f && gx < (float)(a.nx - 1) && gy >= 0.0f && gy < (float)(a.ny - 1) && gz >= 0.0f &&
+                          gz < (float)(a.nz - 1);
+                const float fx0 = floorf(gx), fy0 = floorf(gy), fz0 = floorf(gz);
+                cell.idx = cell.ok ? (int)fx0 + row * (int)fy0 + plane * (int)fz0 : 0;
+                cell.fx = gx - fx0;
+                cell.fy = gy - fy0;
+                cell.fz = gz - fz0;
+            } else {
+                int Y[3], at[3];
+                float F[3], f[3];
+                ref_apply(s_ref, q[p].x, q[p].y, q[p].z, Y, F);
+#pragma unroll
+                for (int r = 0; r < 3; ++r) {
+                    const float g = F[r] + s_b[r];
+                    const float fl = __fadd_rd(g, 12582912.0f);
+                    f[r] = g - (fl - 12582912.0f);
+                    at[r] = __float_as_int(fl) - mg[r] + Y[r];
+                }
+                cell.ok = (unsigned)at[0] < (unsigned)(a.nx - 1) && (unsigned)at[1] < (unsigned)(a.ny - 1) &&
+                          (unsigned)at[2] < (unsigned)(a.nz - 1);
+                cell.idx = at[0] + row * at[1] + plane * at[2];
+                cell.fx = f[0];
+                cell.fy = f[1];
+                cell.fz = f[2];
+            }
+            gather<VARIANT, TS, true>(a, row, plane, cell, s, c);
+        }
+        c = __reduce_add_sync(0xffffffffu, c);
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) {
+            accS[warp] += s;
+            accC[warp] += c;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        float S = 0.0f;
+        int C = 0;
+        for (int w = 0; w < FIT_WARPS; ++w) {
+            S += accS[w];
+            C += accC[w];
+        }
+        a.part_S[by] = S;
+        a.part_C[by] = C;
+        __threadfence();
+        s_last = atomicAdd(a.counter, 1u) == (unsigned)a.n_ptiles - 1;
+    }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    // up to a few hundred tiles: every thread sums tiles tid, tid + 256, ...
+    // and the block combines the sums in a fixed order
+    float S = 0.0f;
+    int C = 0;
+    for (int y = tid; y < a.n_ptiles; y += FIT_THREADS) {
+        S += __ldcg(a.part_S + y);
+        C += __ldcg(a.part_C + y);
+    }
+    for (int o = 16; o > 0; o >>= 1) S += __shfl_xor_sync(0xffffffffu, S, o);
+    C = __reduce_add_sync(0xffffffffu, C);
+    if (lane == 0) {
+        accS[warp] = S;
+        accC[warp] = C;
+    }
+    __syncthreads();
+    if (tid == 0) {
+        *a.counter = 0u;
+        if (!skip) {
+            S = 0.0f;
+            C = 0;
+            for (int w = 0; w < FIT_WARPS; ++w) {
+                S += accS[w];
+                C += accC[w];
+            }
+            const float E = C > 0 ? __fdiv_rn(S, (float)C) : INFINITY;
+            const double e = isfinite(E) ? (double)E : 1.0;
+            scale_search(st, a.beta + (1.0 - a.beta) * e);
+            st->pending_s = 0;
+            a.stats->E_new[a.iter] = E;
+        }
+    }
 }
 
 // One launch over the CTAs of several independent problems (the sequences
@@ -1828,9 +2022,13 @@ constexpr float kParticleLanesBelowCells = 5.0f;
 constexpr float kParticleLanesBelowNodes = 12.0f;
 
 template <int SRC, typename TS>
-void launch_fitness_t(const FitArgs& a, int layout, dim3 grid, cudaStream_t s)
+void launch_fitness_t(const FitArgs& a, int layout, dim3 grid, bool roomy, cudaStream_t s)
 {
-    if (layout == 2)
+    if (roomy && layout == 2)
+        fitness_kernel<SRC, 0, TS, 1><<<grid, FIT_THREADS, 0, s>>>(a);
+    else if (roomy)
+        fitness_kernel<SRC, 2, TS, 1><<<grid, FIT_THREADS, 0, s>>>(a);
+    else if (layout == 2)
         fitness_kernel<SRC, 0, TS><<<grid, FIT_THREADS, 0, s>>>(a);
     else
         fitness_kernel<SRC, 2, TS><<<grid, FIT_THREADS, 0, s>>>(a);
@@ -1852,17 +2050,44 @@ void launch_fitness(FitArgs a, int variant, const pf_volume* v, int chunks, cuda
     const float auto_threshold = layout == 3 ? kParticleLanesBelowCells : kParticleLanesBelowNodes;
     a.pm_threshold = mapping == 1 ? -1.0f : mapping == 2 ? INFINITY : auto_threshold;
     dim3 grid(chunks, a.n_ptiles);
+    const bool roomy = (long long)chunks * a.n_ptiles <= device_sms(v->device);
     const pf_dtype dt = pf_fitness_dtype(v, layout);  // the cell view's records, or the node array's values
     if (layout == 1)  // the plain baseline: float tsdf and weights
         fitness_kernel<SRC, 1, float><<<grid, FIT_THREADS, 0, s>>>(a);
     else if (dt == PF_F16)
-        launch_fitness_t<SRC, __half>(a, layout, grid, s);
+        launch_fitness_t<SRC, __half>(a, layout, grid, roomy, s);
     else if (dt == PF_BF16)
-        launch_fitness_t<SRC, __nv_bfloat16>(a, layout, grid, s);
+        launch_fitness_t<SRC, __nv_bfloat16>(a, layout, grid, roomy, s);
     else if (dt == PF_FP8E4M3)
-        launch_fitness_t<SRC, __nv_fp8_e4m3>(a, layout, grid, s);
+        launch_fitness_t<SRC, __nv_fp8_e4m3>(a, layout, grid, roomy, s);
     else
-        launch_fitness_t<SRC, float>(a, layout, grid, s);
+        launch_fitness_t<SRC, float>(a, layout, grid, roomy, s);
+    pf::count_launch();
+}
+
+template <typename TS>
+void launch_eval_t(const FitArgs& a, int layout, cudaStream_t s)
+{
+    if (layout == 2)
+        search_eval_kernel<0, TS><<<a.n_ptiles, FIT_THREADS, 0, s>>>(a);
+    else
+        search_eval_kernel<2, TS><<<a.n_ptiles, FIT_THREADS, 0, s>>>(a);
+}
+
+void launch_eval(const FitArgs& a, const pf_volume* v, cudaStream_t s)
+{
+    const int layout = resolve_fitness_layout(v);
+    const pf_dtype dt = pf_fitness_dtype(v, layout);
+    if (layout == 1)
+        search_eval_kernel<1, float><<<a.n_ptiles, FIT_THREADS, 0, s>>>(a);
+    else if (dt == PF_F16)
+        launch_eval_t<__half>(a, layout, s);
+    else if (dt == PF_BF16)
+        launch_eval_t<__nv_bfloat16>(a, layout, s);
+    else if (dt == PF_FP8E4M3)
+        launch_eval_t<__nv_fp8_e4m3>(a, layout, s);
+    else
+        launch_eval_t<float>(a, layout, s);
     pf::count_launch();
 }
 
@@ -2168,11 +2393,10 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
         pf::timing_end(pf::KC_FITNESS, s);
         if (p->update_mode == 0) {
             FitArgs e = a;
-            e.chunks = nullptr;  // one particle, built in its CTAs
             e.K = 1;
             e.n_ptiles = choose_ptiles(v->device, 1, ne_max);
             pf::timing_begin(pf::KC_FITNESS1, s);
-            launch_fitness<SRC_EVAL>(e, v->fitness_variant, v, 1, s);
+            launch_eval(e, v, s);
             pf::timing_end(pf::KC_FITNESS1, s);
         }
     }
@@ -2742,6 +2966,8 @@ cudaError_t preload_fitness_storage()
     cudaFuncAttributes fa;
     cudaError_t e = cudaFuncGetAttributes(&fa, fitness_kernel<SRC_POSES, 0, TS>);
     if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fitness_kernel<SRC_POSES, 2, TS>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fitness_kernel<SRC_POSES, 0, TS, 1>);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&fa, fitness_kernel<SRC_POSES, 2, TS, 1>);
     return e;
 }
 
