@@ -10,6 +10,7 @@ not been built.
 from __future__ import annotations
 
 import ctypes as C
+import functools
 import os
 
 import numpy as np
@@ -499,7 +500,10 @@ def backproject(depth, intr, stream=None):
 # autograd
 # ---------------------------------------------------------------------------
 
+@functools.cache
 def _align_function():
+    """The autograd function's class (made on first use: torch is imported
+    then; making it anew for each call took some 50 us of host time)."""
     import torch
 
     class AlignLoss(torch.autograd.Function):
