@@ -27,12 +27,13 @@
 //     inside the grid skips the per-axis range test and forms its cell index
 //     as one linear combination.  A float cell-view record (32 bytes) is one
 //     256-bit load.
-//   * The last CTA to finish (ticket counter, no spinning) reduces the
-//     partials over point tiles and, for the search, does the selection:
-//     argmin (lowest index on ties), advantage set, its mean, the FP64 pose
-//     composition with re-orthonormalisation and the search-size update.
-//     One launch per iteration therefore carries the whole iteration; the
-//     paper's mean update adds one single-particle launch for E(P_new).
+//   * The last CTA of each particle chunk (ticket counters, no spinning)
+//     reduces the chunk's partials over point tiles; search_select_kernel
+//     selects (argmin with the lowest index on ties, advantage set, its mean),
+//     composes the FP64 pose with re-orthonormalisation and updates the search
+//     size; the paper's mean update adds search_eval_kernel for E(P_new).
+//     Launches of pf_fitness and of batches reduce, and the latter select, in
+//     their last CTA.
 //   * Everything stays on the device: a frame is a fixed sequence of
 //     launches with no host round trip, so it can be captured in a graph.
 #include <float.h>
