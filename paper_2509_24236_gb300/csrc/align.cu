@@ -57,6 +57,7 @@ struct AlignScratch {
     double* part = nullptr;       // align partials: frames x tiles x 8 (tiles <= AL_TILES)
     size_t part_cap = 0;          // doubles
     long long* acc = nullptr;     // n_nodes fixed-point dL/dV
+    bool acc_zero = false;        // and it is zero whenever no call is in flight
     double* gn_part = nullptr;    // (AL_TILES + GN_CLASSES) x GN_VALS
     double* gn_state = nullptr;   // see GnState
     void* frame_pose = nullptr;   // frames x FramePose (the poses prepared once per frame)
@@ -968,6 +969,21 @@ AlignScratch& scratch_of(const pf_volume* v)
     return g_scratch[v];
 }
 
+// Zeroes device memory before it returns, on a stream of its own: on the
+// caller's stream, which may be capturing, the fill would only be recorded,
+// and a call before the graph's first launch, or after the graph is dropped,
+// would find the memory as it came.
+cudaError_t zero_now(void* p, size_t bytes)
+{
+    cudaStream_t z = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&z, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, 0, bytes, z);
+    const cudaError_t e2 = cudaStreamSynchronize(z);
+    cudaStreamDestroy(z);
+    return e != cudaSuccess ? e : e2;
+}
+
 }  // namespace
 
 namespace pf {
@@ -1016,15 +1032,11 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
         sc.frame_cap = n_frames;
     }
     // the accumulator is zero between calls: fixed_to_float leaves it so
-    if (grad_tsdf_dev && !sc.acc) {
-        long long* acc = nullptr;
-        PF_CUDA(pf::dev_malloc(&acc, v->n_nodes * sizeof(long long)));
-        const cudaError_t e = cudaMemsetAsync(acc, 0, v->n_nodes * sizeof(long long), s);
-        if (e != cudaSuccess) {
-            cudaFree(acc);
-            return pf::cuda_status(e);
-        }
-        sc.acc = acc;
+    if (grad_tsdf_dev && !sc.acc_zero) {
+        if (!sc.acc) PF_CUDA(pf::dev_malloc(&sc.acc, v->n_nodes * sizeof(long long)));
+        else PF_CUDA(cudaDeviceSynchronize());  // a call that failed half-way may still write to it
+        PF_CUDA(zero_now(sc.acc, v->n_nodes * sizeof(long long)));
+        sc.acc_zero = true;
     }
     AlignArgs a;
     a.tsdf = v->tsdf;
@@ -1051,10 +1063,7 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
         pf::count_launch();
     }
     const cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess && grad_tsdf_dev) {  // the accumulator may not be zero: a new one for the next call
-        cudaFree(sc.acc);
-        sc.acc = nullptr;
-    }
+    if (e != cudaSuccess && grad_tsdf_dev) sc.acc_zero = false;  // (its address may be in a captured graph: kept)
     return pf::cuda_status(e);
 }
 
