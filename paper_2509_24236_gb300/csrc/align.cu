@@ -969,21 +969,6 @@ AlignScratch& scratch_of(const pf_volume* v)
     return g_scratch[v];
 }
 
-// Zeroes device memory before it returns, on a stream of its own: on the
-// caller's stream, which may be capturing, the fill would only be recorded,
-// and a call before the graph's first launch, or after the graph is dropped,
-// would find the memory as it came.
-cudaError_t zero_now(void* p, size_t bytes)
-{
-    cudaStream_t z = nullptr;
-    cudaError_t e = cudaStreamCreateWithFlags(&z, cudaStreamNonBlocking);
-    if (e != cudaSuccess) return e;
-    e = cudaMemsetAsync(p, 0, bytes, z);
-    const cudaError_t e2 = cudaStreamSynchronize(z);
-    cudaStreamDestroy(z);
-    return e != cudaSuccess ? e : e2;
-}
-
 }  // namespace
 
 namespace pf {
@@ -1035,7 +1020,7 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
     if (grad_tsdf_dev && !sc.acc_zero) {
         if (!sc.acc) PF_CUDA(pf::dev_malloc(&sc.acc, v->n_nodes * sizeof(long long)));
         else PF_CUDA(cudaDeviceSynchronize());  // a call that failed half-way may still write to it
-        PF_CUDA(zero_now(sc.acc, v->n_nodes * sizeof(long long)));
+        PF_CUDA(pf::zero_now(sc.acc, v->n_nodes * sizeof(long long)));
         sc.acc_zero = true;
     }
     AlignArgs a;

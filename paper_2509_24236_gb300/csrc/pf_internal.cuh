@@ -231,6 +231,23 @@ inline cudaError_t dev_malloc_async(T** p, size_t bytes, cudaStream_t s)
     return cudaMallocAsync(reinterpret_cast<void**>(p), bytes, s);
 }
 
+// Zeroes device memory before it returns, on a stream of its own.  A fill on
+// the legacy default stream is ordered neither before work on a caller's
+// non-blocking stream nor before the host's next step; one on the caller's
+// stream, which may be capturing, would only be recorded, and a call before the
+// graph's first launch, or after the graph is dropped, would find the memory as
+// it came.
+inline cudaError_t zero_now(void* p, size_t bytes)
+{
+    cudaStream_t z = nullptr;
+    cudaError_t e = cudaStreamCreateWithFlags(&z, cudaStreamNonBlocking);
+    if (e != cudaSuccess) return e;
+    e = cudaMemsetAsync(p, 0, bytes, z);
+    const cudaError_t e2 = cudaStreamSynchronize(z);
+    cudaStreamDestroy(z);
+    return e != cudaSuccess ? e : e2;
+}
+
 enum KernelClass { KC_FITNESS = 0, KC_FITNESS1, KC_INTEGRATE, KC_REFRESH, KC_BACKPROJECT, KC_RAYCAST, KC_COUNT };
 
 // Event bracketing of launches (no-ops unless timing is enabled).

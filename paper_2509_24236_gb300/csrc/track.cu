@@ -2117,7 +2117,7 @@ pf_status grow_partials(pf_volume* v, size_t need)
     PF_CUDA(cudaDeviceSynchronize());
     if (!w.counter) {
         PF_CUDA(pf::dev_malloc(&w.counter, sizeof(unsigned int)));
-        PF_CUDA(cudaMemset(w.counter, 0, sizeof(unsigned int)));
+        PF_CUDA(pf::zero_now(w.counter, sizeof(unsigned int)));
     }
     if ((size_t)w.part_cap < need) {
         cudaFree(w.part_S);
@@ -2183,7 +2183,7 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
         w.chunk_C = nullptr;
         PF_CUDA(pf::dev_malloc(reinterpret_cast<ChunkData**>(&w.chunks), sizeof(ChunkData) * (size_t)chunks_needed));
         PF_CUDA(pf::dev_malloc(&w.chunk_counter, sizeof(unsigned int) * (size_t)chunks_needed));
-        PF_CUDA(cudaMemset(w.chunk_counter, 0, sizeof(unsigned int) * (size_t)chunks_needed));
+        PF_CUDA(pf::zero_now(w.chunk_counter, sizeof(unsigned int) * (size_t)chunks_needed));
         PF_CUDA(pf::dev_malloc(&w.chunk_E, sizeof(float) * KC * (size_t)chunks_needed));
         PF_CUDA(pf::dev_malloc(&w.chunk_C, sizeof(int) * KC * (size_t)chunks_needed));
         w.chunk_cap = chunks_needed;
@@ -2218,13 +2218,13 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
     }
     if (!w.state) {
         PF_CUDA(pf::dev_malloc(reinterpret_cast<SelectPart**>(&w.select), sizeof(SelectPart)));
-        PF_CUDA(cudaMemset(w.select, 0, sizeof(SelectPart)));
+        PF_CUDA(pf::zero_now(w.select, sizeof(SelectPart)));
         PF_CUDA(pf::dev_malloc(&w.state, sizeof(SearchState)));
         PF_CUDA(pf::dev_malloc(&w.n_points, sizeof(int)));
         PF_CUDA(pf::dev_malloc(&w.pose_in, 16 * sizeof(double)));
         PF_CUDA(pf::dev_malloc(&w.pose_out, 16 * sizeof(double)));
         PF_CUDA(pf::dev_malloc(&w.stats, sizeof(pf_track_stats)));
-        PF_CUDA(cudaMemset(w.stats, 0, sizeof(pf_track_stats)));
+        PF_CUDA(pf::zero_now(w.stats, sizeof(pf_track_stats)));
     }
     w.k_cap = std::max(w.k_cap, k_max);
     return PF_OK;
@@ -2595,6 +2595,9 @@ pf_status batch_tables(pf_batch* b, bool tune)
     }
     PF_CUDA(cudaMemcpy(b->d_args, args.data(), args.size() * sizeof(FitArgs), cudaMemcpyHostToDevice));
     PF_CUDA(cudaMemcpy(b->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice));
+    // a copy from pageable memory may still be on its way when it returns, and
+    // a step on a non-blocking stream is not ordered after it
+    PF_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
     return PF_OK;
 }
 
@@ -2717,11 +2720,10 @@ pf_status pf_batch_create(int n, pf_volume* const* vols, const pf_intrinsics* in
     }
     if (st != PF_OK) return fail(st);
     cudaError_t e = pf::dev_malloc(&b->depth, depth_total * sizeof(float));
-    if (e == cudaSuccess) e = cudaMemset(b->depth, 0, depth_total * sizeof(float));
+    if (e == cudaSuccess) e = pf::zero_now(b->depth, depth_total * sizeof(float));
     if (e == cudaSuccess) e = pf::dev_malloc(&b->poses, (size_t)n * 64 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemset(b->poses, 0, (size_t)n * 64 * sizeof(double));
     if (e == cudaSuccess) e = pf::dev_malloc(&b->stats, (size_t)n * sizeof(pf_track_stats));
-    if (e == cudaSuccess) e = cudaMemset(b->stats, 0, (size_t)n * sizeof(pf_track_stats));
+    if (e == cudaSuccess) e = pf::zero_now(b->stats, (size_t)n * sizeof(pf_track_stats));
     if (e == cudaSuccess) e = pf::dev_malloc(&b->tune_state, (size_t)n * sizeof(SearchState));
     if (e == cudaSuccess) e = pf::dev_malloc(&b->tune_stats, (size_t)n * sizeof(pf_track_stats));
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking);

@@ -749,7 +749,7 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     if (e == cudaSuccess && view)
         e = pf::dev_malloc(&v->tile_stamp, sizeof(int) * ((size_t)v->tiles[0] * v->tiles[1] * v->tiles[2] + 1));
     if (e == cudaSuccess && view)
-        e = cudaMemset(v->tile_stamp, 0, sizeof(int) * ((size_t)v->tiles[0] * v->tiles[1] * v->tiles[2] + 1));
+        e = pf::zero_now(v->tile_stamp, sizeof(int) * ((size_t)v->tiles[0] * v->tiles[1] * v->tiles[2] + 1));
     if (e != cudaSuccess) {
         cudaFree(v->tsdf);
         cudaFree(v->weight);
