@@ -2593,6 +2593,8 @@ pf_status batch_tables(pf_batch* b, bool tune)
         PF_CUDA(pf::dev_malloc(&b->d_args, args.size() * sizeof(FitArgs)));
         PF_CUDA(pf::dev_malloc(&b->d_first, first.size() * sizeof(int)));
     }
+    // steps in flight, on whichever stream, read the tables that are rewritten
+    PF_CUDA(cudaDeviceSynchronize());
     PF_CUDA(cudaMemcpy(b->d_args, args.data(), args.size() * sizeof(FitArgs), cudaMemcpyHostToDevice));
     PF_CUDA(cudaMemcpy(b->d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice));
     // a copy from pageable memory may still be on its way when it returns, and
@@ -2811,7 +2813,6 @@ pf_status pf_batch_step(pf_batch* b, void* stream)
 pf_status pf_batch_set_points_per_block(pf_batch* b, int points_per_block)
 {
     if (!b || points_per_block < SUBTILE || points_per_block > (1 << 24)) return PF_ERR_INVALID_ARG;
-    PF_CUDA(cudaDeviceSynchronize());
     b->points_per_block = points_per_block;
     batch_drop_graph(b);
     return batch_tables(b, false);
@@ -2820,7 +2821,6 @@ pf_status pf_batch_set_points_per_block(pf_batch* b, int points_per_block)
 pf_status pf_batch_set_mapping_threshold(pf_batch* b, float voxels)
 {
     if (!b || !(voxels <= 1e6f)) return PF_ERR_INVALID_ARG;
-    PF_CUDA(cudaDeviceSynchronize());
     b->pm_threshold = voxels > 0.0f ? voxels : 0.0f;
     batch_drop_graph(b);
     return batch_tables(b, false);

@@ -6,7 +6,8 @@ stream (PyTorch's streams are such), cudaMemset returns before it has run, and
 a copy from pageable memory may return before it has arrived.  A missing wait
 shows on a GPU only by chance, so the sources are checked: fills go through
 zero_now, which waits, and whatever copies a batch's tables or a volume's nodes
-waits after the last copy."""
+waits after the last copy.  A batch's tables are rewritten only once no step
+that reads them is in flight."""
 import glob
 import os
 import re
@@ -39,3 +40,10 @@ def test_host_copies_are_waited_for():
         assert re.search(r"cuda(Device|Stream)Synchronize\(", text[last:]), name
     create = body(source("track.cu"), "pf_status pf_batch_create(")
     assert create.rindex("cudaMemcpyHostToDevice") < create.index("batch_tables(b, false)")  # which waits
+
+
+def test_batch_tables_are_rewritten_between_steps():
+    tables = body(source("track.cu"), "pf_status batch_tables(")
+    assert tables.index("cudaDeviceSynchronize()") < tables.index("cudaMemcpyHostToDevice")
+    # every change of a table goes through there
+    assert source("track.cu").count("cudaMemcpy(b->d_args") == 1
