@@ -2159,6 +2159,10 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
 {
     if (!v || max_pixels < 1 || k_max < 1) return PF_ERR_INVALID_ARG;
     pf_workspace& w = v->ws;
+    // with what was reserved before: the callers take a frame of up to pix_cap
+    // pixels with up to k_cap particles as reserved, whichever call brought each
+    max_pixels = std::max(max_pixels, w.pix_cap);
+    k_max = std::max(k_max, w.k_cap);
     const long long ne_max = max_pixels;
     // partial slots: the largest tiles x particles over every particle count
     // up to k_max and every point count up to max_pixels
@@ -2226,7 +2230,7 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
         PF_CUDA(pf::dev_malloc(&w.stats, sizeof(pf_track_stats)));
         PF_CUDA(pf::zero_now(w.stats, sizeof(pf_track_stats)));
     }
-    w.k_cap = std::max(w.k_cap, k_max);
+    w.k_cap = k_max;
     return PF_OK;
 }
 
@@ -2301,7 +2305,7 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
     const int npix = intr->width * intr->height;
     pf_workspace& w = v->ws;
     if (w.pix_cap < npix || w.k_cap < p->k_max || !w.state) {
-        st = pf::workspace_reserve(v, std::max(npix, w.pix_cap), std::max(p->k_max, w.k_cap));
+        st = pf::workspace_reserve(v, npix, p->k_max);
         if (st != PF_OK) return st;
     }
     cudaStream_t s = (cudaStream_t)stream;
@@ -2423,7 +2427,7 @@ static pf_status pf_track_frame_impl(pf_volume* v, const float* depth_dev, const
     const int npix = intr->width * intr->height;
     pf_workspace& w = v->ws;
     if (w.pix_cap < npix || w.k_cap < p->k_max || !w.state) {
-        st = pf::workspace_reserve(v, std::max(npix, w.pix_cap), std::max(p->k_max, w.k_cap));
+        st = pf::workspace_reserve(v, npix, p->k_max);
         if (st != PF_OK) return st;
     }
     cudaStream_t s = (cudaStream_t)stream;
@@ -2716,9 +2720,7 @@ pf_status pf_batch_create(int n, pf_volume* const* vols, const pf_intrinsics* in
     };
     pf_status st = PF_OK;
     for (int i = 0; i < n && st == PF_OK; ++i) {
-        pf_workspace& w = vols[i]->ws;
-        st = pf::workspace_reserve(vols[i], std::max(intrs[i].width * intrs[i].height, w.pix_cap),
-                                   std::max(params[i].k_max, w.k_cap));
+        st = pf::workspace_reserve(vols[i], intrs[i].width * intrs[i].height, params[i].k_max);
     }
     if (st != PF_OK) return fail(st);
     cudaError_t e = pf::dev_malloc(&b->depth, depth_total * sizeof(float));
