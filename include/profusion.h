@@ -19,7 +19,9 @@
  *   - Pointers named *_dev are device pointers owned by the caller; *_host
  *     are host pointers owned by the caller.  The library never frees caller
  *     memory.  The library owns the volume's device memory and its workspace
- *     from pf_create_volume until pf_destroy_volume.
+ *     from pf_create_volume until pf_destroy_volume.  A workspace that a later
+ *     call outgrows is kept until then (altogether at most twice the size of
+ *     the present one), so captured graphs and batches that use it stay valid.
  *   - cuda_stream is a cudaStream_t passed as void*; NULL is the legacy
  *     default stream.  All kernels of a call are enqueued on that stream.
  *   - Errors: every call returns pf_status and never aborts.  Arguments are

@@ -1002,19 +1002,16 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
     AlignScratch& sc = scratch_of(v);
     const int tiles = std::max(1, std::min(AL_TILES, (AL_BLOCKS + n_frames - 1) / n_frames));
     const size_t need = (size_t)n_frames * tiles * 8;
+    pf_volume* owner = const_cast<pf_volume*>(v);
     if (sc.part_cap < need) {
-        cudaFree(sc.part);
-        sc.part = nullptr;
-        sc.part_cap = 0;
-        PF_CUDA(pf::dev_malloc(&sc.part, need * sizeof(double)));
-        sc.part_cap = need;
+        const size_t cap = (size_t)pf::grown_capacity((long long)sc.part_cap, (long long)need);
+        PF_CUDA(pf::grow_scratch(owner, {pf::grow(&sc.part, cap)}));
+        sc.part_cap = cap;
     }
     if (sc.frame_cap < n_frames) {
-        cudaFree(sc.frame_pose);
-        sc.frame_pose = nullptr;
-        sc.frame_cap = 0;
-        PF_CUDA(pf::dev_malloc(&sc.frame_pose, (size_t)n_frames * sizeof(FramePose)));
-        sc.frame_cap = n_frames;
+        const int cap = (int)pf::grown_capacity(sc.frame_cap, n_frames);
+        PF_CUDA(pf::grow_scratch(owner, {pf::grow(reinterpret_cast<FramePose**>(&sc.frame_pose), (size_t)cap)}));
+        sc.frame_cap = cap;
     }
     // the accumulator is zero between calls: fixed_to_float leaves it so
     if (grad_tsdf_dev && !sc.acc_zero) {

@@ -9,9 +9,11 @@
 
 #include <atomic>
 #include <cmath>
+#include <vector>
 
 #include "../../include/profusion.h"
 #include "cellpitch.h"
+#include "growbuf.h"
 
 // --------------------------------------------------------------------------
 // TSDF value encoding in the f32 tsdf array.
@@ -189,6 +191,7 @@ struct pf_volume {
     FusionList list;
     SurfaceMap surf;
     pf_workspace ws;
+    std::vector<void*> retired;  // outgrown scratch, kept for the graphs and tables that hold it
 };
 
 // Storage type of the cell view's records: the node array's, or the search
@@ -246,6 +249,31 @@ inline cudaError_t zero_now(void* p, size_t bytes)
     const cudaError_t e2 = cudaStreamSynchronize(z);
     cudaStreamDestroy(z);
     return e != cudaSuccess ? e : e2;
+}
+
+// Replaces scratch buffers of a volume by larger ones (see growbuf.h).
+inline cudaError_t grow_scratch(pf_volume* v, std::initializer_list<Grow> set)
+{
+    const cudaError_t e = grow_all(
+        v->retired, set,
+        [](void** p, size_t bytes, bool zero) {
+            cudaError_t a = dev_malloc(p, bytes);
+            if (a == cudaSuccess && zero) a = zero_now(*p, bytes);
+            if (a != cudaSuccess) {
+                cudaFree(*p);
+                *p = nullptr;
+            }
+            return a;
+        },
+        [](void* p) { cudaFree(p); });
+    if (e != cudaSuccess) cudaGetLastError();  // reported here, not by the next launch
+    return e;
+}
+
+template <typename T>
+inline Grow grow(T** p, size_t count, bool zero = false)
+{
+    return {p, count * sizeof(T), zero};
 }
 
 enum KernelClass { KC_FITNESS = 0, KC_FITNESS1, KC_INTEGRATE, KC_REFRESH, KC_BACKPROJECT, KC_RAYCAST, KC_COUNT };

@@ -2110,26 +2110,34 @@ void fill_volume_args(FitArgs& a, const pf_volume* v, int layout)
     for (int q = 0; q < 3; ++q) a.org[q] = v->desc.origin[q];
 }
 
+// Partial sums for `need` (tile, particle) slots.
 pf_status grow_partials(pf_volume* v, size_t need)
 {
     pf_workspace& w = v->ws;
-    if ((size_t)w.part_cap >= need && w.counter) return PF_OK;
-    PF_CUDA(cudaDeviceSynchronize());
-    if (!w.counter) {
-        PF_CUDA(pf::dev_malloc(&w.counter, sizeof(unsigned int)));
-        PF_CUDA(pf::zero_now(w.counter, sizeof(unsigned int)));
-    }
+    if (!w.counter) PF_CUDA(pf::grow_scratch(v, {pf::grow(&w.counter, 1, true)}));
     if ((size_t)w.part_cap < need) {
-        cudaFree(w.part_S);
-        cudaFree(w.part_C);
-        w.part_S = nullptr;
-        w.part_C = nullptr;
-        w.part_cap = 0;
-        PF_CUDA(pf::dev_malloc(&w.part_S, need * sizeof(float)));
-        PF_CUDA(pf::dev_malloc(&w.part_C, need * sizeof(int)));
-        w.part_cap = (int)need;
+        const size_t cap = (size_t)pf::grown_capacity(w.part_cap, (long long)need);
+        PF_CUDA(pf::grow_scratch(v, {pf::grow(&w.part_S, cap), pf::grow(&w.part_C, cap)}));
+        w.part_cap = (int)cap;
     }
     return PF_OK;
+}
+
+// Buffers for frames of `cap` pixels.
+cudaError_t grow_frame(pf_volume* v, int cap)
+{
+    pf_workspace& w = v->ws;
+    const size_t n = (size_t)cap, slots = kept_slots_bound(n);
+    // one count per back-projection block: an image of n pixels has at most n
+    // tiles (thin images leave tiles partly empty)
+    const cudaError_t e = pf::grow_scratch(
+        v, {pf::grow(&w.points, n), pf::grow(&w.block_counts, n / BP_CHUNK_TILES + 2), pf::grow(&w.point_tile, n),
+            pf::grow(&w.kept, 2 * n), pf::grow(&w.kept_count, 4), pf::grow(&w.order_scratch, 3 * slots)});
+    if (e == cudaSuccess) {
+        w.order_cap = (int)slots;
+        w.pix_cap = cap;
+    }
+    return e;
 }
 
 pf_status check_params(const pf_track_params* p)
@@ -2163,73 +2171,33 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
     // pixels with up to k_cap particles as reserved, whichever call brought each
     max_pixels = std::max(max_pixels, w.pix_cap);
     k_max = std::max(k_max, w.k_cap);
-    const long long ne_max = max_pixels;
+    if (w.pix_cap < max_pixels) {
+        const int cap = (int)std::min(pf::grown_capacity(w.pix_cap, max_pixels), (long long)INT_MAX);
+        cudaError_t e = grow_frame(v, cap);
+        if (e == cudaErrorMemoryAllocation && cap > max_pixels) e = grow_frame(v, max_pixels);
+        if (e != cudaSuccess) return pf::cuda_status(e);
+    }
     // partial slots: the largest tiles x particles over every particle count
-    // up to k_max and every point count up to max_pixels
+    // up to k_max and every point count up to pix_cap
     size_t need = 0;
     for (int chunks = 1; chunks <= (k_max + KC - 1) / KC; ++chunks) {
         const size_t K = std::min((size_t)chunks * KC, (size_t)k_max);
-        need = std::max(need, (size_t)ptiles_bound(v->device, chunks, ne_max) * K);
+        need = std::max(need, (size_t)ptiles_bound(v->device, chunks, w.pix_cap) * K);
     }
     pf_status st = grow_partials(v, need);
     if (st != PF_OK) return st;
     const int chunks_needed = (k_max + KC - 1) / KC;
     if (w.chunk_cap < chunks_needed) {
-        PF_CUDA(cudaDeviceSynchronize());
-        cudaFree(w.chunks);
-        w.chunks = nullptr;
-        w.chunk_cap = 0;
-        cudaFree(w.chunk_counter);
-        cudaFree(w.chunk_E);
-        cudaFree(w.chunk_C);
-        w.chunk_counter = nullptr;
-        w.chunk_E = nullptr;
-        w.chunk_C = nullptr;
-        PF_CUDA(pf::dev_malloc(reinterpret_cast<ChunkData**>(&w.chunks), sizeof(ChunkData) * (size_t)chunks_needed));
-        PF_CUDA(pf::dev_malloc(&w.chunk_counter, sizeof(unsigned int) * (size_t)chunks_needed));
-        PF_CUDA(pf::zero_now(w.chunk_counter, sizeof(unsigned int) * (size_t)chunks_needed));
-        PF_CUDA(pf::dev_malloc(&w.chunk_E, sizeof(float) * KC * (size_t)chunks_needed));
-        PF_CUDA(pf::dev_malloc(&w.chunk_C, sizeof(int) * KC * (size_t)chunks_needed));
-        w.chunk_cap = chunks_needed;
+        const size_t cap = (size_t)pf::grown_capacity(w.chunk_cap, chunks_needed);
+        PF_CUDA(pf::grow_scratch(v, {pf::grow(reinterpret_cast<ChunkData**>(&w.chunks), cap),
+                                     pf::grow(&w.chunk_counter, cap, true), pf::grow(&w.chunk_E, KC * cap),
+                                     pf::grow(&w.chunk_C, KC * cap)}));
+        w.chunk_cap = (int)cap;
     }
-    if (w.pix_cap < max_pixels) {
-        PF_CUDA(cudaDeviceSynchronize());
-        cudaFree(w.points);
-        cudaFree(w.block_counts);
-        cudaFree(w.point_tile);
-        cudaFree(w.kept);
-        cudaFree(w.kept_count);
-        cudaFree(w.order_scratch);
-        w.points = nullptr;
-        w.block_counts = nullptr;
-        w.point_tile = nullptr;
-        w.kept = nullptr;
-        w.kept_count = nullptr;
-        w.order_scratch = nullptr;
-        w.order_cap = 0;
-        w.pix_cap = 0;
-        PF_CUDA(pf::dev_malloc(&w.point_tile, sizeof(int) * (size_t)max_pixels));
-        PF_CUDA(pf::dev_malloc(&w.kept, 2 * sizeof(float4) * (size_t)max_pixels));
-        PF_CUDA(pf::dev_malloc(&w.kept_count, 4 * sizeof(int)));
-        const size_t slots = kept_slots_bound((size_t)max_pixels);
-        PF_CUDA(pf::dev_malloc(&w.order_scratch, 3 * sizeof(int) * slots));
-        w.order_cap = (int)slots;
-        PF_CUDA(pf::dev_malloc(&w.points, sizeof(float4) * (size_t)max_pixels));
-        // one count per back-projection block: an image of max_pixels pixels has
-        // at most max_pixels tiles (thin images leave tiles partly empty)
-        PF_CUDA(pf::dev_malloc(&w.block_counts, sizeof(int) * ((size_t)max_pixels / BP_CHUNK_TILES + 2)));
-        w.pix_cap = max_pixels;
-    }
-    if (!w.state) {
-        PF_CUDA(pf::dev_malloc(reinterpret_cast<SelectPart**>(&w.select), sizeof(SelectPart)));
-        PF_CUDA(pf::zero_now(w.select, sizeof(SelectPart)));
-        PF_CUDA(pf::dev_malloc(&w.state, sizeof(SearchState)));
-        PF_CUDA(pf::dev_malloc(&w.n_points, sizeof(int)));
-        PF_CUDA(pf::dev_malloc(&w.pose_in, 16 * sizeof(double)));
-        PF_CUDA(pf::dev_malloc(&w.pose_out, 16 * sizeof(double)));
-        PF_CUDA(pf::dev_malloc(&w.stats, sizeof(pf_track_stats)));
-        PF_CUDA(pf::zero_now(w.stats, sizeof(pf_track_stats)));
-    }
+    if (!w.state)
+        PF_CUDA(pf::grow_scratch(v, {pf::grow(reinterpret_cast<SelectPart**>(&w.select), 1, true),
+                                     pf::grow(reinterpret_cast<SearchState**>(&w.state), 1), pf::grow(&w.n_points, 1),
+                                     pf::grow(&w.pose_in, 16), pf::grow(&w.pose_out, 16), pf::grow(&w.stats, 1, true)}));
     w.k_cap = k_max;
     return PF_OK;
 }
@@ -2467,6 +2435,10 @@ struct pf_batch {
     std::vector<size_t> depth_off;
     double* poses = nullptr;
     pf_track_stats* stats = nullptr;
+    // the point buffers that the launch tables name (a volume's workspace may
+    // have grown into others since)
+    std::vector<float4*> points;
+    std::vector<int*> block_counts;
     // launch tables, per iteration: arguments of every participating
     // sequence and the first CTA of each (search, then single-pose
     // evaluation for the mean update)
@@ -2542,9 +2514,13 @@ FitArgs batch_args(const pf_batch* b, int i, SearchState* st, pf_track_stats* st
 pf_status batch_tables(pf_batch* b, bool tune)
 {
     const int n = b->n, iters = b->max_iters;
-    // partial slots each volume needs over all iterations, grown first (a
-    // reallocation would leave stale pointers in earlier table entries)
+    // partial slots each volume needs over all iterations, grown first (the
+    // entries of all iterations name the same ones)
+    std::vector<float4*> points(n);
+    std::vector<int*> block_counts(n);
     for (int i = 0; i < n; ++i) {
+        points[i] = b->vols[i]->ws.points;
+        block_counts[i] = b->vols[i]->ws.block_counts;
         const pf_track_params& p = b->params[i];
         const long long npix = (long long)b->intrs[i].width * b->intrs[i].height;
         size_t need = 0;
@@ -2604,6 +2580,8 @@ pf_status batch_tables(pf_batch* b, bool tune)
     // a copy from pageable memory may still be on its way when it returns, and
     // a step on a non-blocking stream is not ordered after it
     PF_CUDA(cudaStreamSynchronize(cudaStreamLegacy));
+    b->points = points;
+    b->block_counts = block_counts;
     return PF_OK;
 }
 
@@ -2647,7 +2625,7 @@ pf_status batch_enqueue(pf_batch* b, cudaStream_t s)
         track_begin_kernel<<<1, 32, 0, s>>>(reinterpret_cast<SearchState*>(v->ws.state), b->init(i),
                                             b->params[i].init_rot_deg, b->params[i].init_trans_cm, b->stats + i);
         pf::count_launch();
-        st = enqueue_backproject(b->depth + b->depth_off[i], &b->intrs[i], v->ws.points, v->ws.block_counts,
+        st = enqueue_backproject(b->depth + b->depth_off[i], &b->intrs[i], b->points[i], b->block_counts[i],
                                  v->ws.n_points, s);
         if (st != PF_OK) return st;
     }

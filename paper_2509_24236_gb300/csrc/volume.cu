@@ -803,6 +803,7 @@ pf_status pf_destroy_volume(pf_volume* v)
     cudaFree(w.pose_in);
     cudaFree(w.pose_out);
     cudaFree(w.stats);
+    for (void* p : v->retired) cudaFree(p);
     delete v;
     return PF_OK;
 }
