@@ -177,6 +177,7 @@ struct SurfaceMap {
 struct pf_volume {
     pf_volume_desc desc;
     int device = 0;
+    int sms = 0;               // of the device (calls of other volumes run in other threads: no shared cache)
     size_t n_nodes = 0;
     void* tsdf = nullptr;      // encoded, see above; float, half or bfloat16 (desc.tsdf_dtype)
     void* weight = nullptr;    // float, or uint8 when desc.weight_u8

@@ -1994,27 +1994,16 @@ __global__ void track_end_kernel(const SearchState* st, const int* n_points, dou
     }
 }
 
-int device_sms(int dev)
-{
-    static int cached_dev = -1, cached_n = 0;
-    if (dev == cached_dev) return cached_n;
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 152;
-    cached_dev = dev;
-    cached_n = n;
-    return n;
-}
-
 // Point tiles of a launch (the rule and its bound: ptiles.h), for this
 // device's resident CTA slots.
-int choose_ptiles(int dev, int chunks, long long ne_max)
+int choose_ptiles(const pf_volume* v, int chunks, long long ne_max)
 {
-    return pf::choose_ptiles_for((long long)device_sms(dev) * PF_FIT_MIN_BLOCKS, SUBTILE, chunks, ne_max);
+    return pf::choose_ptiles_for((long long)v->sms * PF_FIT_MIN_BLOCKS, SUBTILE, chunks, ne_max);
 }
 
-int ptiles_bound(int dev, int chunks, long long ne_max)
+int ptiles_bound(const pf_volume* v, int chunks, long long ne_max)
 {
-    return pf::ptiles_bound_for((long long)device_sms(dev) * PF_FIT_MIN_BLOCKS, SUBTILE, chunks, ne_max);
+    return pf::ptiles_bound_for((long long)v->sms * PF_FIT_MIN_BLOCKS, SUBTILE, chunks, ne_max);
 }
 
 // variant = layout + 4 * mapping (see pf_set_fitness_variant).  Measured on
@@ -2053,7 +2042,7 @@ void launch_fitness(FitArgs a, int variant, const pf_volume* v, int chunks, cuda
     const float auto_threshold = layout == 3 ? kParticleLanesBelowCells : kParticleLanesBelowNodes;
     a.pm_threshold = mapping == 1 ? -1.0f : mapping == 2 ? INFINITY : auto_threshold;
     dim3 grid(chunks, a.n_ptiles);
-    const bool roomy = (long long)chunks * a.n_ptiles <= device_sms(v->device);
+    const bool roomy = (long long)chunks * a.n_ptiles <= v->sms;
     const pf_dtype dt = pf_fitness_dtype(v, layout);  // the cell view's records, or the node array's values
     if (layout == 1)  // the plain baseline: float tsdf and weights
         fitness_kernel<SRC, 1, float><<<grid, FIT_THREADS, 0, s>>>(a);
@@ -2182,7 +2171,7 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
     size_t need = 0;
     for (int chunks = 1; chunks <= (k_max + KC - 1) / KC; ++chunks) {
         const size_t K = std::min((size_t)chunks * KC, (size_t)k_max);
-        need = std::max(need, (size_t)ptiles_bound(v->device, chunks, w.pix_cap) * K);
+        need = std::max(need, (size_t)ptiles_bound(v, chunks, w.pix_cap) * K);
     }
     pf_status st = grow_partials(v, need);
     if (st != PF_OK) return st;
@@ -2230,7 +2219,7 @@ static pf_status pf_fitness_impl(const pf_volume* cv, const float* points_dev, i
     if (!v || !poses_dev || !fitness_dev || !count_dev) return PF_ERR_INVALID_ARG;
     if (n < 0 || k < 1 || k > 65536 || (n > 0 && !points_dev)) return PF_ERR_INVALID_ARG;
     const int chunks = (k + KC - 1) / KC;
-    const int tiles = choose_ptiles(v->device, chunks, n);
+    const int tiles = choose_ptiles(v, chunks, n);
     pf_status st = grow_partials(v, (size_t)tiles * k);
     if (st != PF_OK) return st;
     FitArgs a;
@@ -2347,7 +2336,7 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
                 a.stride = 1;
             }
         a.iter = it;
-        a.n_ptiles = choose_ptiles(v->device, chunks, ne_max);
+        a.n_ptiles = choose_ptiles(v, chunks, ne_max);
         if ((size_t)a.n_ptiles * K > (size_t)w.part_cap || chunks > w.chunk_cap) return PF_ERR_INVALID_ARG;
         // the iteration's particles, built once (the plain baseline layout
         // builds its own in every CTA, as it always did)
@@ -2369,7 +2358,7 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
         if (p->update_mode == 0) {
             FitArgs e = a;
             e.K = 1;
-            e.n_ptiles = choose_ptiles(v->device, 1, ne_max);
+            e.n_ptiles = choose_ptiles(v, 1, ne_max);
             pf::timing_begin(pf::KC_FITNESS1, s);
             launch_eval(e, v, s);
             pf::timing_end(pf::KC_FITNESS1, s);
@@ -2427,7 +2416,6 @@ struct pf_batch {
     int max_iters = 0;
     int layout = 3;
     pf_dtype dtype = PF_F32;
-    int device = 0;
     // device buffers: depth images (one allocation), per sequence four poses
     // (relative input, current pose, initial pose of the search, spare) and
     // the search record
@@ -2481,7 +2469,7 @@ float mapping_threshold(const pf_volume* v, int layout)
 int batch_tiles(const pf_batch* b, int K, long long ne_max)
 {
     const long long max_tiles = std::max(1LL, (ne_max + SUBTILE - 1) / SUBTILE);
-    long long t = K == 1 ? (long long)device_sms(b->device) * 8 : (ne_max + b->points_per_block - 1) / b->points_per_block;
+    long long t = K == 1 ? (long long)b->vols[0]->sms * 8 : (ne_max + b->points_per_block - 1) / b->points_per_block;
     return (int)std::max(1LL, std::min(t, max_tiles));
 }
 
@@ -2684,7 +2672,6 @@ pf_status pf_batch_create(int n, pf_volume* const* vols, const pf_intrinsics* in
     b->params.assign(params, params + n);
     b->layout = resolve_layout(vols[0]);
     b->dtype = pf_fitness_dtype(vols[0], b->layout);
-    b->device = vols[0]->device;
     b->use_graph = use_graph != 0;
     size_t depth_total = 0;
     for (int i = 0; i < n; ++i) {
@@ -3004,7 +2991,7 @@ static pf_status pf_fitness_noalloc_impl(const pf_volume* v, const float* points
     if (st != PF_OK) return st;
     const int chunks = (k + KC - 1) / KC;
     // as many point tiles as pf_fitness would use, within the fixed scratch
-    const int tiles = std::max(1, std::min(choose_ptiles(v->device, chunks, n), PF_NOALLOC_MAX_SLOTS / k));
+    const int tiles = std::max(1, std::min(choose_ptiles(v, chunks, n), PF_NOALLOC_MAX_SLOTS / k));
     FitArgs a;
     memset(&a, 0, sizeof(a));
     a.pts = reinterpret_cast<const float4*>(points_dev);

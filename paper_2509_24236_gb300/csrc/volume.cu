@@ -518,12 +518,7 @@ __global__ void __launch_bounds__(TX * TY, 4) cells_refresh_kernel(RefreshArgs a
 }
 
 // CTAs of the list-walking fusion and refresh kernels: 4 per SM.
-int list_ctas(int device)
-{
-    int sms = 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device) != cudaSuccess || sms <= 0) sms = 152;
-    return 4 * sms;
-}
+int list_ctas(const pf_volume* v) { return 4 * v->sms; }
 
 pf_status enqueue_refresh(pf_volume* v, cudaStream_t s, int all)
 {
@@ -549,7 +544,7 @@ pf_status enqueue_refresh(pf_volume* v, cudaStream_t s, int all)
     }
     refresh_tiles_kernel<<<(n_tiles + 255) / 256, 256, 0, s>>>(r);
     pf::count_launch();
-    const int grid = list_ctas(v->device);
+    const int grid = list_ctas(v);
     const dim3 blk(TX, TY);
     if (v->desc.tsdf_dtype != pf_view_dtype(v)) {  // the search view of a float grid
         switch (pf_view_dtype(v)) {
@@ -643,7 +638,7 @@ pf_status enqueue_surface_scan(pf_volume* v, cudaStream_t s)
     const int n_tiles = v->tiles[0] * v->tiles[1] * v->tiles[2];
     const dim3 blk(TX, TY);
     auto scan = [&](auto kernel) {
-        kernel<<<list_ctas(v->device), blk, 0, s>>>(v->tsdf, v->desc.nx, v->desc.ny, v->desc.nz, v->tiles[0],
+        kernel<<<list_ctas(v), blk, 0, s>>>(v->tsdf, v->desc.nx, v->desc.ny, v->desc.nz, v->tiles[0],
                                                     v->tiles[1], n_tiles, v->surf);
     };
     switch (v->desc.tsdf_dtype) {
@@ -715,6 +710,7 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     const size_t view_bytes = n_cells * 8 * vs;
     const size_t grid_bytes = v->n_nodes * (ts + ws);
     cudaError_t e = cudaGetDevice(&v->device);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&v->sms, cudaDevAttrMultiProcessorCount, v->device);
     int mode = desc->cell_view;
     if (mode == 0) {
         // auto, within half of the device memory free now: the full view
@@ -967,7 +963,7 @@ pf_status integrate_impl(pf_volume* v, const float* depth_dev, const pf_intrinsi
     fusion_begin_kernel<<<PF_DEPTH_BLOCKS * PF_DEPTH_BLOCKS / BEGIN_WARPS, 32 * BEGIN_WARPS, 0, s>>>(
         v->list, v->tile_stamp ? v->tile_stamp + n_tiles : nullptr, depth_dev, a.cam);
     fusion_tiles_kernel<<<(n_tiles + 255) / 256, 256, 0, s>>>(a);
-    dispatch_storage<IntegrateLaunch>(v, list_ctas(v->device), a, s);
+    dispatch_storage<IntegrateLaunch>(v, list_ctas(v), a, s);
     pf::count_launch(3);
     pf::timing_end(pf::KC_INTEGRATE, s);
     PF_LAUNCHED();
