@@ -1422,9 +1422,13 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
             }
             if (!s_mode) {
                 // four particles at a time, so that one transposed butterfly
-                // serves their four sums (fold); one at a time in a batched
-                // launch, whose arguments in shared memory take the registers
-                // (224 bytes of spills otherwise, a mixed batch 3% slower)
+                // serves their four sums (fold); one at a time where that
+                // would spill: in a batched launch, whose arguments in shared
+                // memory take the registers (224 bytes, a mixed batch 3%
+                // slower), and on e4m3 nodes, whose eight decoded bytes a cell
+                // do (248 bytes; 512 poses x 300 000 points of a 256^3 grid
+                // without a view, lanes on points: 991 us, one at a time 865)
+                constexpr bool FOLD = SOLO && (CTAS == 1 || VARIANT != 0 || sizeof(TS) != 1);
                 auto particle = [&](auto checked, int kk, float& s, int& c) {
                     XformD X;
                     load_xformd(sPD[kk], X);
@@ -1443,7 +1447,7 @@ __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, u
                 };
                 auto particles = [&](auto checked) {
                     int kk = 0;
-                    for (; SOLO && kk + 4 <= kc; kk += 4) {
+                    for (; FOLD && kk + 4 <= kc; kk += 4) {
                         float s, half = 0.0f, prev = 0.0f;
                         unsigned c4 = 0u;
 #pragma unroll
