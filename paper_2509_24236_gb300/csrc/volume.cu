@@ -9,12 +9,12 @@
 // GB300 layout: tiles of 32 x 8 x 8 nodes (x fastest, so a warp touches one
 // 128-byte line of each array per slice); a tile is dropped before any memory
 // access when its box lies outside the view frustum, beyond depth_max + tau or
-// behind every depth of the pixels it covers.  Node loads and stores happen
-// only for nodes that pass every test, so HBM traffic is proportional to the
-// nodes actually updated.  The camera-frame depth of a node is formed as a
-// double-precision tile base (split into a float pair) plus a small float
-// offset, which keeps the signed distance accurate to ~1e-7 m at any
-// distance from the grid origin.
+// (in grids of many tiles) behind every depth of the pixels it covers.  Node
+// loads and stores happen only for nodes that pass every test, so HBM traffic
+// is proportional to the nodes actually updated.  The camera-frame depth of a
+// node is formed as a double-precision tile base (split into a float pair)
+// plus a small float offset, which keeps the signed distance accurate to
+// ~1e-7 m at any distance from the grid origin.
 #include <stdlib.h>
 #include <string.h>
 
@@ -57,10 +57,10 @@ struct IntegArgs {
 
 // Starts a fusion: empties the tile lists and, with a cell view, advances the
 // fusion counter the tile stamps refer to (on the device, so a captured and
-// replayed launch sequence still marks each fusion apart).  The fusion's own
-// launch also reduces the image to its blocks' largest usable depths (0: none),
-// one warp a block, for the occlusion cull below; without an image (a refresh
-// outside a fusion) one CTA only empties the lists.
+// replayed launch sequence still marks each fusion apart).  The launch of a
+// fusion with the depth cull also reduces the image to its blocks' largest
+// usable depths (0: none), one warp a block; without an image one CTA only
+// empties the lists.
 constexpr int BEGIN_WARPS = 8;
 
 __global__ void __launch_bounds__(32 * BEGIN_WARPS) fusion_begin_kernel(FusionList list, int* stamp_counter,
@@ -94,6 +94,7 @@ __global__ void __launch_bounds__(32 * BEGIN_WARPS) fusion_begin_kernel(FusionLi
 // many blocks is kept without a look.
 __device__ inline bool tile_occluded(const IntegArgs& a, const float* c, const float* e)
 {
+    if (!a.list.depth_max) return false;
     const float zn = c[2] - e[2], zf = c[2] + e[2];
     if (!(zn > 0.0f)) return false;
     // pixel bounds of the box over its depth range, one pixel wider
@@ -116,7 +117,7 @@ __device__ inline bool tile_occluded(const IntegArgs& a, const float* c, const f
 }
 
 // One thread per fusion tile of TX x TY x TZ nodes: two culls of the tile's
-// box, by the frustum and by the image's depths, and for a tile
+// box, by the frustum and (large grids) by the image's depths, and for a tile
 // that survives the camera-frame position of its first node,
 // X_c = R^T (X_w - t) with X_w = origin + vs (i0, j0, k0), in FP64 -- kept as
 // floats, the depth as a hi + lo pair -- which is appended to the list (its
@@ -738,7 +739,8 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     if (e == cudaSuccess) e = pf::dev_malloc(&v->list.tile, n_tiles * sizeof(int));
     if (e == cudaSuccess) e = pf::dev_malloc(&v->list.base, n_tiles * sizeof(float4));
     if (e == cudaSuccess) e = pf::dev_malloc(&v->list.step, 9 * sizeof(float));
-    if (e == cudaSuccess) e = pf::dev_malloc(&v->list.depth_max, PF_DEPTH_BLOCKS * PF_DEPTH_BLOCKS * sizeof(float));
+    if (e == cudaSuccess && n_tiles > PF_DEPTH_CULL_TILES)
+        e = pf::dev_malloc(&v->list.depth_max, PF_DEPTH_BLOCKS * PF_DEPTH_BLOCKS * sizeof(float));
     if (e == cudaSuccess && view) e = pf::dev_malloc(&v->list.rows, n_tiles * sizeof(unsigned long long));
     if (e == cudaSuccess && view) e = pf::dev_malloc(&v->list.refresh_tile, n_tiles * sizeof(int));
     if (e == cudaSuccess && view) e = pf::dev_malloc(&v->list.refresh_rows, n_tiles * sizeof(unsigned long long));
@@ -960,8 +962,12 @@ pf_status integrate_impl(pf_volume* v, const float* depth_dev, const pf_intrinsi
     a.surf = v->surf;
     ++v->stamp;
     pf::timing_begin(pf::KC_INTEGRATE, s);
-    fusion_begin_kernel<<<PF_DEPTH_BLOCKS * PF_DEPTH_BLOCKS / BEGIN_WARPS, 32 * BEGIN_WARPS, 0, s>>>(
-        v->list, v->tile_stamp ? v->tile_stamp + n_tiles : nullptr, depth_dev, a.cam);
+    int* stamp = v->tile_stamp ? v->tile_stamp + n_tiles : nullptr;
+    if (v->list.depth_max)
+        fusion_begin_kernel<<<PF_DEPTH_BLOCKS * PF_DEPTH_BLOCKS / BEGIN_WARPS, 32 * BEGIN_WARPS, 0, s>>>(v->list, stamp,
+                                                                                                  depth_dev, a.cam);
+    else
+        fusion_begin_kernel<<<1, 32, 0, s>>>(v->list, stamp, nullptr, a.cam);
     fusion_tiles_kernel<<<(n_tiles + 255) / 256, 256, 0, s>>>(a);
     dispatch_storage<IntegrateLaunch>(v, list_ctas(v), a, s);
     pf::count_launch(3);
