@@ -90,7 +90,8 @@ typedef enum { PF_F32 = 0, PF_F16 = 1, PF_BF16 = 2, PF_FP8E4M3 = 3 } pf_dtype;
  * A float grid's records are 32 bytes per node.  The full view of a 16-bit
  * (8-bit) grid keeps a 16-byte (8-byte) record and a 32-byte float record
  * per node; its narrow view keeps the 16-byte (8-byte) record only (lanes
- * on particles then convert on load).  -1 = no view; 1 = the full view;
+ * on particles then convert on load).  (Rows and planes of records may be
+ * padded, which adds at most a sixteenth.)  -1 = no view; 1 = the full view;
  * 2 = the narrow view (a float grid takes 1); 0 = automatic: the full
  * view when the whole volume (grid, weights, view) fits in half of the
  * device memory free at creation (decoding narrow records on load slows the

@@ -31,7 +31,11 @@ struct CellPitch {
 // so nx - 1 records a row suffice and the pitched view of a grid of equal
 // sides fits in the nx * ny * nz records an unpitched one has.  A grid whose
 // pitched view would pass 2^31 records keeps the node grid's pitch (record
-// indices are 32-bit).
+// indices are 32-bit), and so does one whose pitched view would need over a
+// sixteenth more records than it has nodes: grids four to a dozen nodes wide,
+// whose rows would grow by up to half.
+inline CellPitch node_pitch(int nx, int ny, int nz) { return {nx, nx * ny, (long long)nx * ny * nz}; }
+
 inline CellPitch cell_pitch(int nx, int ny, int nz)
 {
     const long long nodes = (long long)nx * ny * nz;
@@ -39,8 +43,29 @@ inline CellPitch cell_pitch(int nx, int ny, int nz)
     const long long rows = row * (ny - 1);
     const long long plane = rows + ((3 - rows) & 3);
     const long long last = (long long)(nx - 2) + row * (ny - 2) + plane * (nz - 2);
-    if (last + 1 >= 2147483648LL) return {nx, nx * ny, nodes};
+    if (last + 1 >= 2147483648LL || last + 1 > nodes + nodes / 16) return node_pitch(nx, ny, nz);
     return {(int)row, (int)plane, last + 1 > nodes ? last + 1 : nodes};
+}
+
+// The cell view of a volume: 1 the full view, 2 the narrow one, -1 none.
+struct CellView {
+    int mode;
+    CellPitch pitch;
+};
+
+// Automatic choice within `budget` bytes, for a grid and weights of grid_bytes
+// and records of narrow_bytes, with wide_bytes more each in the full view (0:
+// the two views are the same): the full view when it fits, else the narrow one,
+// else none.  The node pitch stands in where the pitched view misses the budget
+// and it does not, so the pitch decides no view away.
+inline CellView choose_view(int nx, int ny, int nz, long long grid_bytes, long long narrow_bytes, long long wide_bytes,
+                            long long budget)
+{
+    const CellPitch pitches[2] = {cell_pitch(nx, ny, nz), node_pitch(nx, ny, nz)};
+    for (int mode = 1; mode <= (wide_bytes ? 2 : 1); ++mode)
+        for (const CellPitch& p : pitches)
+            if (grid_bytes + p.count * (narrow_bytes + (mode == 1 ? wide_bytes : 0)) <= budget) return {mode, p};
+    return {-1, pitches[0]};
 }
 
 }  // namespace pf

@@ -705,31 +705,41 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     // on points: two or four records per sector) and float records (lanes on
     // particles: no conversions); the narrow view keeps the narrow records
     // only; a float grid has the float records only
-    v->pitch = pf::cell_pitch(desc->nx, desc->ny, desc->nz);
-    const size_t n_cells = (size_t)v->pitch.count;
-    const size_t bytes32 = vdt == PF_F32 ? 0 : n_cells * 32;
-    const size_t view_bytes = n_cells * 8 * vs;
-    const size_t grid_bytes = v->n_nodes * (ts + ws);
+    const size_t rec = 8 * vs, rec32 = vdt == PF_F32 ? 0 : 32;
+    pf::CellView cv = {desc->cell_view, pf::cell_pitch(desc->nx, desc->ny, desc->nz)};
     cudaError_t e = cudaGetDevice(&v->device);
     if (e == cudaSuccess) e = cudaDeviceGetAttribute(&v->sms, cudaDevAttrMultiProcessorCount, v->device);
-    int mode = desc->cell_view;
-    if (mode == 0) {
+    if (cv.mode == 0) {
         // auto, within half of the device memory free now: the full view
         // when it fits (decoding narrow records on load slows the search
         // once the particles converge), else the narrow one, else none
         size_t free_b = 0, total_b = 0;
         if (e == cudaSuccess) e = cudaMemGetInfo(&free_b, &total_b);
-        const size_t budget = free_b / 2;
-        mode = grid_bytes + view_bytes + bytes32 <= budget ? 1 : grid_bytes + view_bytes <= budget ? 2 : -1;
+        cv = pf::choose_view(desc->nx, desc->ny, desc->nz, (long long)(v->n_nodes * (ts + ws)), (long long)rec,
+                             (long long)rec32, (long long)(free_b / 2));
     }
-    if (mode == 2 && !bytes32) mode = 1;
-    if (mode == -1 && vdt != desc->tsdf_dtype) e = cudaErrorMemoryAllocation;  // no room for the search view
-    const bool view = mode >= 1;
-    const bool wide = mode == 1;
+    if (cv.mode == 2 && !rec32) cv.mode = 1;
+    if (cv.mode == -1 && vdt != desc->tsdf_dtype) e = cudaErrorMemoryAllocation;  // no room for the search view
+    const bool view = cv.mode >= 1;
+    const bool wide = cv.mode == 1 && rec32;
     if (e == cudaSuccess) e = pf::dev_malloc(&v->tsdf, v->n_nodes * ts);
     if (e == cudaSuccess) e = pf::dev_malloc(&v->weight, v->n_nodes * ws);
-    if (e == cudaSuccess && view) e = pf::dev_malloc(&v->cells, view_bytes);
-    if (e == cudaSuccess && wide && bytes32) e = pf::dev_malloc(&v->cells32, bytes32);
+    auto alloc_view = [&]() {
+        cudaError_t a = pf::dev_malloc(&v->cells, (size_t)cv.pitch.count * rec);
+        if (a == cudaSuccess && wide) a = pf::dev_malloc(&v->cells32, (size_t)cv.pitch.count * rec32);
+        return a;
+    };
+    if (e == cudaSuccess && view) {
+        e = alloc_view();
+        if (e == cudaErrorMemoryAllocation && cv.pitch.count > (long long)v->n_nodes) {  // with the node pitch, then
+            cudaGetLastError();
+            cudaFree(v->cells);
+            v->cells = nullptr;
+            cv.pitch = pf::node_pitch(desc->nx, desc->ny, desc->nz);
+            e = alloc_view();
+        }
+    }
+    v->pitch = cv.pitch;
     v->surf.wx = (desc->nx + 31) / 32;
     v->surf.wy = (desc->ny + 31) / 32;
     v->surf.wz = (desc->nz + 31) / 32;
