@@ -31,9 +31,10 @@
 //     b = sum J^T r, sum r^2 and the count for the state's candidate pose
 //     (float per thread, FP64 across threads and tiles); the last block of
 //     the launch accepts the candidate if it lowers the mean squared residual
-//     (lambda /= 10) or drops it (lambda *= 10), solves (H + lambda diag H) d = -b and forms the next
-//     candidate [Exp(d_omega) | d_v] T.  No host round trip: a polish is a
-//     fixed launch sequence.
+//     (lambda /= 10) or drops it (lambda *= 10), solves
+//     (H + lambda diag H) d = -b and forms the next candidate
+//     [Exp(d_omega) | d_v] T.  No host round trip: a polish is a fixed launch
+//     sequence.
 #include <algorithm>
 #include <climits>
 #include <mutex>
@@ -739,8 +740,6 @@ __device__ inline void gn_step(const GnArgs& a, bool evaluated, GnShared& sh)
             if (a.mode == 1) {
                 lambda = take ? lambda / 10.0 : lambda * 10.0;
                 accepted += take;
-            } else if (!take) {
-                lambda *= 10.0;
             }
         }
         const int step = st->step + (a.mode == 1 ? 1 : 0);

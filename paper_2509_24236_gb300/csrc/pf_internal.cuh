@@ -191,7 +191,6 @@ struct pf_volume {
     void* cells = nullptr;     // cell view: a record of 8 values per cell, pitched as `pitch` says
     float* cells32 = nullptr;  // 16-/8-bit grids, full view: the same records as floats (x-differences formed)
     int* tile_stamp = nullptr; // per fusion tile: stamp of the last fusion that reached it
-    int stamp = 0;             // fusions so far
     int tiles[3] = {0, 0, 0};
     pf::CellPitch pitch = {0, 0, 0};  // of the records in cells and cells32
     int fitness_variant = 0;

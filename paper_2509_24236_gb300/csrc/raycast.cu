@@ -18,15 +18,20 @@
 // before each run of them (the crossing needs its value).  Every sample that
 // is evaluated is the one the plain march evaluates, at the same rounded
 // depth, so the results are the same bits.
-// Measured, 640x480 into 512^3: 308 -> 52 us with normals; fusing a frame into 768^3
-// half precision and casting 160x120 of it: 1081 -> 459 us.
+// Measured, 640x480 of an uploaded 512^3 room with normals, the same view again
+// and again: 308 -> 52 us; each time a view not cast before, of a 512^3 map while
+// 100 distinct views are fused into it: 372 -> 128 us for the last 50 (768^3
+// half precision 599 -> 155).  A map whose set bricks consist mostly of cells
+// with an unobserved corner is the one kind that loses: the plain march's first
+// load told it so, here come a lookup and eight loads (64^3, solid, half of the
+// nodes unobserved at random: 48 -> 62 us).  Loading that corner first took 2 to
+// 8% more for every other map, and 53 to 60 us there.
 #include "pf_internal.cuh"
 
 namespace {
 
 struct RayArgs {
     const void* tsdf;
-    const void* weight;
     int nx, ny, nz;
     float inv_vs;
     float org[3];
@@ -197,7 +202,6 @@ static pf_status pf_raycast_impl(const pf_volume* v, const pf_intrinsics* intr, 
         if (!std::isfinite(P[q])) return PF_ERR_INVALID_ARG;
     RayArgs a;
     a.tsdf = v->tsdf;
-    a.weight = v->weight;
     a.nx = v->desc.nx;
     a.ny = v->desc.ny;
     a.nz = v->desc.nz;

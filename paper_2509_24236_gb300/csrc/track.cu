@@ -344,10 +344,12 @@ struct FitArgs {
     const float* poses;   // SRC_POSES: K x 12
     float pm_threshold;   // particles on lanes when the chunk's spread (voxels) is below this
     const float* templ;   // SRC_SEARCH: templates, row k = particle k
-    const void* chunks;   // the launch's particle chunks built by chunk_build_kernel, or null: each CTA builds its own
-    // search of one problem: the last CTA of each chunk writes its particles'
-    // E and count here, search_select_kernel selects (a batched launch's last
+    // Search of one problem: the particle chunks that chunk_build_kernel built
+    // (layouts 2 and 3; with the plain layout, in batches and in pf_fitness each
+    // CTA builds its own), and where the last CTA of each chunk writes its
+    // particles' E and count for search_select_kernel (a batched launch's last
     // CTA reduces every particle over the point tiles and selects)
+    const void* chunks;
     unsigned int* chunk_counter;
     float* chunk_E;
     int* chunk_C;
@@ -447,7 +449,7 @@ struct Particle {      // shared memory, 64 bytes
 constexpr int kMagicBits = 0x4b400000;  // bits of 1.5 * 2^23
 constexpr int kNeverValid = 0x7fffffff;  // magic of a particle that reaches no cell
 
-// Camera-to-world pose of particle k in FP64.
+// Camera-to-world pose of particle k in FP64 (SRC_POSES, SRC_SEARCH).
 template <int SRC, bool SERIES = false>
 __device__ inline void particle_pose(const FitArgs& a, int k, double R[9], double tw[3])
 {
@@ -459,24 +461,16 @@ __device__ inline void particle_pose(const FitArgs& a, int k, double R[9], doubl
         }
     } else {
         const double* P = a.st->P;
-        if (SRC == SRC_EVAL) {
-            for (int r = 0; r < 3; ++r) {
-                for (int c = 0; c < 3; ++c) R[3 * r + c] = P[4 * r + c];
-                tw[r] = P[4 * r + 3];
-            }
-        } else {
-            const float* u = a.templ + 6 * (size_t)k;
-            const double wr = a.st->w[0], wt = a.st->w[1];
-            const double dw[3] = {wr * (double)u[0], wr * (double)u[1], wr * (double)u[2]};
-            double dR[9];
-            so3_exp_d<SERIES>(dw, dR);
-            for (int r = 0; r < 3; ++r) {
-                for (int c = 0; c < 3; ++c)
-                    R[3 * r + c] = dR[3 * r] * P[c] + dR[3 * r + 1] * P[4 + c] + dR[3 * r + 2] * P[8 + c];
-                const double tr = a.compose_mode == 0 ? dR[3 * r] * P[3] + dR[3 * r + 1] * P[7] + dR[3 * r + 2] * P[11]
-                                                      : P[4 * r + 3];
-                tw[r] = tr + wt * (double)u[3 + r];
-            }
+        const float* u = a.templ + 6 * (size_t)k;
+        const double wr = a.st->w[0], wt = a.st->w[1];
+        const double dw[3] = {wr * (double)u[0], wr * (double)u[1], wr * (double)u[2]};
+        double dR[9];
+        so3_exp_d<SERIES>(dw, dR);
+        for (int r = 0; r < 3; ++r) {
+            for (int c = 0; c < 3; ++c) R[3 * r + c] = dR[3 * r] * P[c] + dR[3 * r + 1] * P[4 + c] + dR[3 * r + 2] * P[8 + c];
+            const double tr =
+                a.compose_mode == 0 ? dR[3 * r] * P[3] + dR[3 * r + 1] * P[7] + dR[3 * r + 2] * P[11] : P[4 * r + 3];
+            tw[r] = tr + wt * (double)u[3 + r];
         }
     }
 }
@@ -810,7 +804,8 @@ __device__ __forceinline__ int linear_cell(const int* Yi, int nx, int nxy)
 // add the same two numbers) and so the same bits.  With fold<16> of values 0
 // and 1 and of 2 and 3, then fold<8> of the two, the lane ends up with value
 // folded_index(lane).  Shuffles go through the L1 data pipe that bounds lanes on
-// points: 3072 spread poses over 307 200 points 5% faster (3.42 -> 3.25 ms).
+// points: 3072 poses 3 degrees apart over 307 200 points of a room's 512^3 grid,
+// sampled as perf/cases.py does, 3.42 -> 3.25 ms.
 template <int O>
 __device__ __forceinline__ float fold(float v0, float v1, int lane)
 {
@@ -903,8 +898,8 @@ static_assert(sizeof(ChunkData) % 16 == 0, "ChunkData is copied as 16-byte words
 
 // Particles k_begin .. k_begin + kc - 1 (kc <= 32) as a CTA uses them, by one
 // warp: lane t builds particle t against the chunk's first, and the chunk's
-// spread and reach are warp reductions.  With sAbs, also each particle's plain
-// float transform.  SERIES: the series form of the exponential.
+// spread and reach are warp reductions.  With sAbs (never for SRC_EVAL), also
+// each particle's plain float transform.  SERIES: the series form of the exponential.
 // FP64 instructions, a hundred cycles of latency and more apiece, are what it
 // costs (conversions to and from FP64 are such too), so they are counted: the
 // scale 1 / vs and the search size come ready, the first particle's products
@@ -922,7 +917,7 @@ __device__ void build_chunk(const FitArgs& a, int k_begin, int kc, ChunkData& C,
     double A0 = 0.0;  // lane q < 9: element q of the first particle's matrix in grid units
     double tg[3];
     bool ok = true;
-    if (SRC == SRC_EVAL) {
+    if constexpr (SRC == SRC_EVAL) {
         // the one particle is its own reference: its matrix differs by zero
         const double* P = a.st->P;
         if (t < 9) A0 = P[4 * (t / 3) + t % 3] * a.iv;
@@ -950,7 +945,7 @@ __device__ void build_chunk(const FitArgs& a, int k_begin, int kc, ChunkData& C,
         const double o = ok ? floor(tg[r]) : 0.0;
         row[r].w = (float)(tg[r] - o);
         m[r] = kMagicBits - (int)o;
-        if (sAbs && mine) sAbs[t].c[r] = (float)tg[r];
+        if (SRC != SRC_EVAL && sAbs && mine) sAbs[t].c[r] = (float)tg[r];
     }
     if (!ok) m[0] = kNeverValid;
     if (mine) {
@@ -1243,9 +1238,10 @@ __global__ void __launch_bounds__(64) search_select_kernel(FitArgs a)
 // The work of one CTA: particle chunk bx, point tile by, of a launch of
 // n_blocks CTAs for this problem (the last of them to finish runs the
 // epilogue).
-// SOLO: a launch of one problem, which may use prebuilt particle chunks and
-// the two-level reduction (FitArgs.chunks, .chunk_counter); the batched
-// launch compiles without them.
+// SOLO: a launch of one problem.  Its search takes the prebuilt particle chunks
+// (layouts 2 and 3), reduces each chunk in the chunk's last CTA and leaves the
+// selection to search_select_kernel, so FitArgs.chunks, .chunk_counter, .chunk_E
+// and .chunk_C must be set; the batched launch compiles without these.
 // CTAS: see fitness_kernel.
 template <int SRC, int VARIANT, typename TS, bool SOLO, int CTAS = PF_FIT_MIN_BLOCKS>
 __device__ __forceinline__ void fitness_body(const FitArgs& a, int bx, int by, unsigned n_blocks)
@@ -2345,7 +2341,7 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
         // the iteration's particles, built once (the plain baseline layout
         // builds its own in every CTA, as it always did)
         const bool prebuild = resolve_fitness_layout(v) != 1;
-        a.chunks = prebuild ? w.chunks : nullptr;
+        a.chunks = w.chunks;
         a.chunk_counter = w.chunk_counter;
         a.chunk_E = w.chunk_E;
         a.chunk_C = w.chunk_C;
