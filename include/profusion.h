@@ -380,10 +380,9 @@ PF_API pf_status pf_batch_tuning(const pf_batch* batch, int* points_per_block, f
  * preparation and the sums across warps and thread blocks are FP64; dL/dV is
  * accumulated in 2^-40 fixed point (int64).  The first call allocates library scratch
  * (n_frames x 2368 doubles; with grad_tsdf_dev also n_nodes x 8 bytes) kept
- * until the volume is destroyed.  Asynchronous on cuda_stream, but for the
- * first call with grad_tsdf_dev, which waits until its scratch is zero (on a
- * stream of its own, so a capture of cuda_stream that permits allocation may
- * hold that call too). */
+ * until the volume is destroyed.  Asynchronous on cuda_stream.  A capture that
+ * permits allocation may hold the first call with grad_tsdf_dev too (its
+ * scratch is then zeroed at once, on another stream, which is waited for). */
 PF_API pf_status pf_align_loss(const pf_volume* vol, const float* points_dev, const int* counts_dev, int n_max,
                                int n_frames, const double* poses_dev, const double* xi_dev, const double* dloss_dev,
                                double* loss_dev, int* count_dev, double* grad_xi_dev, float* grad_tsdf_dev,

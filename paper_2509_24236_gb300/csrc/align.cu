@@ -1004,19 +1004,19 @@ static pf_status pf_align_loss_impl(const pf_volume* v, const float* points_dev,
     pf_volume* owner = const_cast<pf_volume*>(v);
     if (sc.part_cap < need) {
         const size_t cap = (size_t)pf::grown_capacity((long long)sc.part_cap, (long long)need);
-        PF_CUDA(pf::grow_scratch(owner, {pf::grow(&sc.part, cap)}));
+        PF_CUDA(pf::grow_scratch(owner, {pf::grow(&sc.part, cap)}, &s));
         sc.part_cap = cap;
     }
     if (sc.frame_cap < n_frames) {
         const int cap = (int)pf::grown_capacity(sc.frame_cap, n_frames);
-        PF_CUDA(pf::grow_scratch(owner, {pf::grow(reinterpret_cast<FramePose**>(&sc.frame_pose), (size_t)cap)}));
+        PF_CUDA(pf::grow_scratch(owner, {pf::grow(reinterpret_cast<FramePose**>(&sc.frame_pose), (size_t)cap)}, &s));
         sc.frame_cap = cap;
     }
     // the accumulator is zero between calls: fixed_to_float leaves it so
     if (grad_tsdf_dev && !sc.acc_zero) {
         if (!sc.acc) PF_CUDA(pf::dev_malloc(&sc.acc, v->n_nodes * sizeof(long long)));
         else PF_CUDA(cudaDeviceSynchronize());  // a call that failed half-way may still write to it
-        PF_CUDA(pf::zero_now(sc.acc, v->n_nodes * sizeof(long long)));
+        PF_CUDA(pf::zero_for(sc.acc, v->n_nodes * sizeof(long long), &s));
         sc.acc_zero = true;
     }
     AlignArgs a;

@@ -2100,20 +2100,20 @@ void fill_volume_args(FitArgs& a, const pf_volume* v, int layout)
 }
 
 // Partial sums for `need` (tile, particle) slots.
-pf_status grow_partials(pf_volume* v, size_t need)
+pf_status grow_partials(pf_volume* v, size_t need, const cudaStream_t* s)
 {
     pf_workspace& w = v->ws;
-    if (!w.counter) PF_CUDA(pf::grow_scratch(v, {pf::grow(&w.counter, 1, true)}));
+    if (!w.counter) PF_CUDA(pf::grow_scratch(v, {pf::grow(&w.counter, 1, true)}, s));
     if ((size_t)w.part_cap < need) {
         const size_t cap = (size_t)pf::grown_capacity(w.part_cap, (long long)need);
-        PF_CUDA(pf::grow_scratch(v, {pf::grow(&w.part_S, cap), pf::grow(&w.part_C, cap)}));
+        PF_CUDA(pf::grow_scratch(v, {pf::grow(&w.part_S, cap), pf::grow(&w.part_C, cap)}, s));
         w.part_cap = (int)cap;
     }
     return PF_OK;
 }
 
 // Buffers for frames of `cap` pixels.
-cudaError_t grow_frame(pf_volume* v, int cap)
+cudaError_t grow_frame(pf_volume* v, int cap, const cudaStream_t* s)
 {
     pf_workspace& w = v->ws;
     const size_t n = (size_t)cap, slots = kept_slots_bound(n);
@@ -2121,7 +2121,8 @@ cudaError_t grow_frame(pf_volume* v, int cap)
     // tiles (thin images leave tiles partly empty)
     const cudaError_t e = pf::grow_scratch(
         v, {pf::grow(&w.points, n), pf::grow(&w.block_counts, n / BP_CHUNK_TILES + 2), pf::grow(&w.point_tile, n),
-            pf::grow(&w.kept, 2 * n), pf::grow(&w.kept_count, 4), pf::grow(&w.order_scratch, 3 * slots)});
+            pf::grow(&w.kept, 2 * n), pf::grow(&w.kept_count, 4), pf::grow(&w.order_scratch, 3 * slots)},
+        s);
     if (e == cudaSuccess) {
         w.order_cap = (int)slots;
         w.pix_cap = cap;
@@ -2152,7 +2153,7 @@ pf_status check_params(const pf_track_params* p)
 
 namespace pf {
 
-pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
+pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max, const cudaStream_t* s)
 {
     if (!v || max_pixels < 1 || k_max < 1) return PF_ERR_INVALID_ARG;
     pf_workspace& w = v->ws;
@@ -2162,8 +2163,8 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
     k_max = std::max(k_max, w.k_cap);
     if (w.pix_cap < max_pixels) {
         const int cap = (int)std::min(pf::grown_capacity(w.pix_cap, max_pixels), (long long)INT_MAX);
-        cudaError_t e = grow_frame(v, cap);
-        if (e == cudaErrorMemoryAllocation && cap > max_pixels) e = grow_frame(v, max_pixels);
+        cudaError_t e = grow_frame(v, cap, s);
+        if (e == cudaErrorMemoryAllocation && cap > max_pixels) e = grow_frame(v, max_pixels, s);
         if (e != cudaSuccess) return pf::cuda_status(e);
     }
     // partial slots: the largest tiles x particles over every particle count
@@ -2173,20 +2174,21 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max)
         const size_t K = std::min((size_t)chunks * KC, (size_t)k_max);
         need = std::max(need, (size_t)ptiles_bound(v, chunks, w.pix_cap) * K);
     }
-    pf_status st = grow_partials(v, need);
+    pf_status st = grow_partials(v, need, s);
     if (st != PF_OK) return st;
     const int chunks_needed = (k_max + KC - 1) / KC;
     if (w.chunk_cap < chunks_needed) {
         const size_t cap = (size_t)pf::grown_capacity(w.chunk_cap, chunks_needed);
         PF_CUDA(pf::grow_scratch(v, {pf::grow(reinterpret_cast<ChunkData**>(&w.chunks), cap),
                                      pf::grow(&w.chunk_counter, cap, true), pf::grow(&w.chunk_E, KC * cap),
-                                     pf::grow(&w.chunk_C, KC * cap)}));
+                                     pf::grow(&w.chunk_C, KC * cap)}, s));
         w.chunk_cap = (int)cap;
     }
     if (!w.state)
         PF_CUDA(pf::grow_scratch(v, {pf::grow(reinterpret_cast<SelectPart**>(&w.select), 1, true),
                                      pf::grow(reinterpret_cast<SearchState**>(&w.state), 1), pf::grow(&w.n_points, 1),
-                                     pf::grow(&w.pose_in, 16), pf::grow(&w.pose_out, 16), pf::grow(&w.stats, 1, true)}));
+                                     pf::grow(&w.pose_in, 16), pf::grow(&w.pose_out, 16), pf::grow(&w.stats, 1, true)},
+                                 s));
     w.k_cap = k_max;
     return PF_OK;
 }
@@ -2220,7 +2222,8 @@ static pf_status pf_fitness_impl(const pf_volume* cv, const float* points_dev, i
     if (n < 0 || k < 1 || k > 65536 || (n > 0 && !points_dev)) return PF_ERR_INVALID_ARG;
     const int chunks = (k + KC - 1) / KC;
     const int tiles = choose_ptiles(v, chunks, n);
-    pf_status st = grow_partials(v, (size_t)tiles * k);
+    cudaStream_t s = (cudaStream_t)stream;
+    pf_status st = grow_partials(v, (size_t)tiles * k, &s);
     if (st != PF_OK) return st;
     FitArgs a;
     memset(&a, 0, sizeof(a));
@@ -2237,7 +2240,6 @@ static pf_status pf_fitness_impl(const pf_volume* cv, const float* points_dev, i
     a.n_ptiles = tiles;
     a.out_E = fitness_dev;
     a.out_C = count_dev;
-    cudaStream_t s = (cudaStream_t)stream;
     pf::timing_begin(pf::KC_FITNESS, s);
     launch_fitness<SRC_POSES>(a, v->fitness_variant, v, chunks, s);
     pf::timing_end(pf::KC_FITNESS, s);
@@ -2247,7 +2249,7 @@ static pf_status pf_fitness_impl(const pf_volume* cv, const float* points_dev, i
 
 static pf_status pf_track_reserve_impl(pf_volume* v, int max_pixels, int k_max)
 {
-    return pf::workspace_reserve(v, max_pixels, k_max);
+    return pf::workspace_reserve(v, max_pixels, k_max, nullptr);
 }
 
 static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev, const pf_intrinsics* intr,
@@ -2261,11 +2263,11 @@ static pf_status pf_track_frame_async_impl(pf_volume* v, const float* depth_dev,
     if (st != PF_OK) return st;
     const int npix = intr->width * intr->height;
     pf_workspace& w = v->ws;
+    cudaStream_t s = (cudaStream_t)stream;
     if (w.pix_cap < npix || w.k_cap < p->k_max || !w.state) {
-        st = pf::workspace_reserve(v, npix, p->k_max);
+        st = pf::workspace_reserve(v, npix, p->k_max, &s);
         if (st != PF_OK) return st;
     }
-    cudaStream_t s = (cudaStream_t)stream;
     pf_track_stats* stats = stats_dev ? stats_dev : w.stats;
     SearchState* state = reinterpret_cast<SearchState*>(w.state);
 
@@ -2383,11 +2385,11 @@ static pf_status pf_track_frame_impl(pf_volume* v, const float* depth_dev, const
     if (st != PF_OK) return st;
     const int npix = intr->width * intr->height;
     pf_workspace& w = v->ws;
+    cudaStream_t s = (cudaStream_t)stream;
     if (w.pix_cap < npix || w.k_cap < p->k_max || !w.state) {
-        st = pf::workspace_reserve(v, npix, p->k_max);
+        st = pf::workspace_reserve(v, npix, p->k_max, &s);
         if (st != PF_OK) return st;
     }
-    cudaStream_t s = (cudaStream_t)stream;
     PF_CUDA(cudaMemcpyAsync(w.pose_in, init_pose, 16 * sizeof(double), cudaMemcpyHostToDevice, s));
     st = pf_track_frame_async(v, depth_dev, intr, p, w.pose_in, w.pose_out, w.stats, stream);
     if (st != PF_OK) return st;
@@ -2518,7 +2520,7 @@ pf_status batch_tables(pf_batch* b, bool tune)
             need = std::max(need, (size_t)batch_tiles(b, p.k_sched[it % 3], ne_max) * p.k_sched[it % 3]);
             need = std::max(need, (size_t)batch_tiles(b, 1, ne_max));
         }
-        pf_status st = grow_partials(b->vols[i], need);
+        pf_status st = grow_partials(b->vols[i], need, nullptr);
         if (st != PF_OK) return st;
     }
     std::vector<FitArgs> args((size_t)iters * 2 * n);
@@ -2685,7 +2687,7 @@ pf_status pf_batch_create(int n, pf_volume* const* vols, const pf_intrinsics* in
     };
     pf_status st = PF_OK;
     for (int i = 0; i < n && st == PF_OK; ++i) {
-        st = pf::workspace_reserve(vols[i], intrs[i].width * intrs[i].height, params[i].k_max);
+        st = pf::workspace_reserve(vols[i], intrs[i].width * intrs[i].height, params[i].k_max, nullptr);
     }
     if (st != PF_OK) return fail(st);
     cudaError_t e = pf::dev_malloc(&b->depth, depth_total * sizeof(float));

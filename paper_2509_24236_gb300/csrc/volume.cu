@@ -696,6 +696,7 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     *out = nullptr;
     pf_status st = check_desc(desc);
     if (st != PF_OK) return st;
+    cudaStream_t s = (cudaStream_t)stream;
     pf_volume* v = new pf_volume();
     v->desc = *desc;
     v->n_nodes = (size_t)desc->nx * desc->ny * desc->nz;
@@ -761,7 +762,7 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
     if (e == cudaSuccess && view)
         e = pf::dev_malloc(&v->tile_stamp, sizeof(int) * ((size_t)v->tiles[0] * v->tiles[1] * v->tiles[2] + 1));
     if (e == cudaSuccess && view)
-        e = pf::zero_now(v->tile_stamp, sizeof(int) * ((size_t)v->tiles[0] * v->tiles[1] * v->tiles[2] + 1));
+        e = pf::zero_for(v->tile_stamp, sizeof(int) * ((size_t)v->tiles[0] * v->tiles[1] * v->tiles[2] + 1), &s);
     if (e != cudaSuccess) {
         cudaFree(v->tsdf);
         cudaFree(v->weight);
@@ -774,7 +775,7 @@ pf_status pf_create_volume(const pf_volume_desc* desc, void* stream, pf_volume**
         cudaGetLastError();
         return pf::cuda_status(e);
     }
-    st = enqueue_reset(v, (cudaStream_t)stream);
+    st = enqueue_reset(v, s);
     if (st != PF_OK) {
         pf_destroy_volume(v);
         return st;
