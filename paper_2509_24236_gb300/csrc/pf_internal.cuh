@@ -264,7 +264,10 @@ inline cudaError_t zero_now(void* p, size_t bytes)
 inline cudaError_t zero_for(void* p, size_t bytes, const cudaStream_t* s)
 {
     cudaStreamCaptureStatus c = cudaStreamCaptureStatusActive;
-    if (s && cudaStreamIsCapturing(*s, &c) != cudaSuccess) cudaGetLastError();
+    if (s && cudaStreamIsCapturing(*s, &c) != cudaSuccess) {  // the legacy stream beside a capture
+        cudaGetLastError();
+        c = cudaStreamCaptureStatusActive;
+    }
     return s && c == cudaStreamCaptureStatusNone ? cudaMemsetAsync(p, 0, bytes, *s) : zero_now(p, bytes);
 }
 

@@ -3,9 +3,8 @@ call finds zero.  Made inside a stream capture it must be zero all the same for
 calls that run before the graph's first launch, and when the graph is dropped.
 
 The memory that the accumulator is given is filled beforehand: blocks of its
-size (256 KiB, which the driver cuts from a larger piece and hands out as they
-are), written by other volumes and freed.  So a fill that was only recorded
-shows."""
+size (256 KiB, which CUDA cuts from a larger piece and hands out as they are),
+written by other volumes and freed.  So a fill that was only recorded shows."""
 import numpy as np
 import pytest
 
