@@ -2161,18 +2161,14 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max, const cudaS
     // pixels with up to k_cap particles as reserved, whichever call brought each
     max_pixels = std::max(max_pixels, w.pix_cap);
     k_max = std::max(k_max, w.k_cap);
-    if (w.pix_cap < max_pixels) {
-        const int cap = (int)std::min(pf::grown_capacity(w.pix_cap, max_pixels), (long long)INT_MAX);
-        cudaError_t e = grow_frame(v, cap, s);
-        if (e == cudaErrorMemoryAllocation && cap > max_pixels) e = grow_frame(v, max_pixels, s);
-        if (e != cudaSuccess) return pf::cuda_status(e);
-    }
+    // (pix_cap and k_cap, which the callers ask, rise when all the rest is there)
+    const int cap_pixels = (int)std::min(pf::grown_capacity(w.pix_cap, max_pixels), (long long)INT_MAX);
     // partial slots: the largest tiles x particles over every particle count
-    // up to k_max and every point count up to pix_cap
+    // up to k_max and every point count up to cap_pixels
     size_t need = 0;
     for (int chunks = 1; chunks <= (k_max + KC - 1) / KC; ++chunks) {
         const size_t K = std::min((size_t)chunks * KC, (size_t)k_max);
-        need = std::max(need, (size_t)ptiles_bound(v, chunks, w.pix_cap) * K);
+        need = std::max(need, (size_t)ptiles_bound(v, chunks, cap_pixels) * K);
     }
     pf_status st = grow_partials(v, need, s);
     if (st != PF_OK) return st;
@@ -2189,6 +2185,11 @@ pf_status workspace_reserve(pf_volume* v, int max_pixels, int k_max, const cudaS
                                      pf::grow(reinterpret_cast<SearchState**>(&w.state), 1), pf::grow(&w.n_points, 1),
                                      pf::grow(&w.pose_in, 16), pf::grow(&w.pose_out, 16), pf::grow(&w.stats, 1, true)},
                                  s));
+    if (w.pix_cap < cap_pixels) {
+        cudaError_t e = grow_frame(v, cap_pixels, s);
+        if (e == cudaErrorMemoryAllocation && cap_pixels > max_pixels) e = grow_frame(v, max_pixels, s);
+        if (e != cudaSuccess) return pf::cuda_status(e);
+    }
     w.k_cap = k_max;
     return PF_OK;
 }
